@@ -139,6 +139,26 @@ int upload_thresholds(Context *c, System &s)
     build_thresholds(s, s.thr_pinned);
     CUDA_TRY(c, cudaMemcpyAsync((void *)s.p.thr, s.thr_pinned, s.thr_count * sizeof(uint32_t),
                                 cudaMemcpyHostToDevice, c->stream));
+    if (s.p.thrT) CUDA_TRY(c, mucal::launch_thr_transpose(s.p, c->stream));
+    return MUCAL_OK;
+}
+
+// The dE-major table copies that multi-commit rounds with thresholds in
+// global memory read: allocated when a launch shape first needs them, kept
+// up to date by upload_thresholds from then on.
+int ensure_thr_transposed(Context *c)
+{
+    for (auto &s : c->sys) {
+        if (s.p.thrT) continue;
+        const int pitch = (s.p.n_bins + 2 * mucal::kThrTPad + 3) & ~3;
+        const size_t bytes = (size_t)s.p.width * (size_t)pitch * sizeof(uint32_t);
+        void *ptr = nullptr;
+        CUDA_TRY(c, cudaMalloc(&ptr, bytes));
+        s.p.thrT = static_cast<const uint32_t *>(ptr);
+        s.p.thrT_pitch = pitch;
+        CUDA_TRY(c, cudaMemsetAsync(ptr, 0, bytes, c->stream));
+        CUDA_TRY(c, mucal::launch_thr_transpose(s.p, c->stream));
+    }
     return MUCAL_OK;
 }
 
@@ -297,6 +317,7 @@ void free_system(System &s)
     cudaFree(s.p.E);
     cudaFree(s.p.hist);
     cudaFree((void *)s.p.thr);
+    cudaFree((void *)s.p.thrT);
     cudaFree(s.p.accepts);
     cudaFree(s.p.H);
     if (s.thr_pinned) cudaFreeHost(s.thr_pinned);
@@ -345,7 +366,7 @@ size_t smem_for(const LaunchShape &sh, const SysParams &p)
     else if (sh.bits_in_smem)
         bytes += (size_t)sh.walkers_per_block * (size_t)p.words * sizeof(uint32_t);
     // the windows start on the next 16-byte boundary behind the bitsets or fields
-    if (!sh.thr_in_smem && sh.thr_window && sh.kernel != MUCAL_KERNEL_THREAD)
+    if (!sh.thr_in_smem && (sh.thr_window || sh.scan_window) && sh.kernel != MUCAL_KERNEL_THREAD)
         bytes += 16 + (size_t)sh.walkers_per_block * mucal::thr_window_bytes(p);
     return bytes;
 }
@@ -460,12 +481,119 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
     if (smem > (size_t)c->max_smem)
         return fail(c, MUCAL_ERR_INVALID_ARG, "launch needs %zu bytes of shared memory, limit %d",
                     smem, c->max_smem);
-    if (!sh.thr_in_smem && sh.thr_window) sh.multi_commit = 0;   // rounds read row windows
+    if (!sh.thr_in_smem && sh.thr_window) sh.multi_commit = 0;   // one-commit rounds read row windows
+    if (sh.multi_commit && !sh.thr_in_smem) {
+        // rounds with several commits keep windows of their own where they fit
+        sh.scan_window = 1;
+        size_t with = 0;
+        for (auto &s : c->sys) with = std::max(with, smem_for(sh, s.p));
+        if (with <= (size_t)c->max_smem) smem = with;
+        else sh.scan_window = 0;
+    }
     sh.smem_bytes = smem;
+    if (sh.multi_commit && !sh.thr_in_smem && !sh.scan_window) {
+        const int rc = ensure_thr_transposed(c);
+        if (rc != MUCAL_OK) return rc;
+    }
     int rc = build_work(c, sh);
     if (rc != MUCAL_OK) return rc;
     c->shape = sh;
     return MUCAL_OK;
+}
+
+// The launch shape of a new context: several commits per round, 8 lanes per
+// walker, on count fields or on the bitsets.
+//
+// A walker is a serial chain, so what counts is that all walkers run at once,
+// or in equal waves, with as many of them beside each other on an SM as its
+// shared memory holds.  One system: its walkers per SM are split into the
+// fewest waves that fit, one block per SM and wave.  Measured on GB300 (ms of
+// the walker update, 16 walkers per block against this rule): 2D L = 64,
+// N = 410, 4096 walkers, 50 sweeps 3.75 -> 3.11 (28 walkers, one wave); 3D
+// L = 32, N = 3277, 8192 walkers, 10 sweeps 13.4 -> 12.8 (28, two waves); 2D
+// L = 74, N = 100, 1024 walkers, 137 sweeps 1.81 -> 1.77 (8, one wave).  Where
+// blocks of 4, 8, 12... walkers at 8 lanes need a wave more than blocks of
+// 2, 4, 6... at 16 lanes, 16 lanes: 3D L = 48, N = 11059, 2048 walkers,
+// 4 sweeps 14.1 (12 walkers, two waves) -> 6.7 (14, one wave).  Several
+// systems: small blocks, which pack their uneven bitsets and lengths best
+// (the 27-system batch, 5 sweeps: 8 walkers 12.4, 4 walkers 10.8).
+//
+// Fields (two byte loads per attempt instead of 4d words, 4d more atomics per
+// commit) where they fit 16 walkers to a block and do not cost a resident
+// walker: 2D L = 64 3.24 (bitsets) -> 3.11, but five 2D systems of L = 61 to
+// 97, 5120 walkers, 50 sweeps 1.10 (bitsets) against 1.95.
+mucal_launch_config default_launch(Context *c)
+{
+    long long total = 0;
+    for (auto &s : c->sys) total += s.p.n_walkers;
+    int sms = 1;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    const long long need = (total + sms - 1) / sms;     // walkers per SM
+    auto fits = [&](int kernel, int lanes, int w, int bits) {
+        LaunchShape sh{};
+        sh.kernel = kernel;
+        sh.lanes = lanes;
+        sh.walkers_per_block = w;
+        sh.bits_in_smem = bits;
+        sh.thr_in_smem = 1;
+        bool table = true, window = true;
+        for (auto &s : c->sys) table = table && smem_for(sh, s.p) <= (size_t)c->max_smem;
+        if (table) return true;
+        sh.thr_in_smem = 0;
+        sh.scan_window = 1;
+        for (auto &s : c->sys) window = window && smem_for(sh, s.p) <= (size_t)c->max_smem;
+        return window;
+    };
+    auto plain_fits = [&](int kernel) {
+        bool ok = true;
+        LaunchShape sh{};
+        sh.kernel = kernel;
+        sh.lanes = 8;
+        sh.walkers_per_block = 16;
+        sh.bits_in_smem = 1;
+        for (auto &s : c->sys) ok = ok && smem_for(sh, s.p) <= (size_t)c->max_smem;
+        return ok;
+    };
+    mucal_launch_config def{MUCAL_KERNEL_GROUP, 8, 16, 1, 0, 0, 1};
+    if (!plain_fits(MUCAL_KERNEL_GROUP) && !fits(MUCAL_KERNEL_GROUP, 8, 4, 1)) {
+        def.bits_in_smem = 0;
+        return def;
+    }
+    // the most walkers a block can hold (an SM's, at one block per SM)
+    auto most = [&](int kernel, int lanes) {
+        const int step = 32 / lanes;
+        int w = 0;
+        while ((w + step) * lanes <= 512 && fits(kernel, lanes, w + step, 1)) w += step;
+        return w;
+    };
+    int cap8 = most(MUCAL_KERNEL_GROUP, 8);
+    if (plain_fits(MUCAL_KERNEL_FIELD)) {
+        const int f = most(MUCAL_KERNEL_FIELD, 8);
+        if (f >= need || f >= cap8) {
+            def.kernel = MUCAL_KERNEL_FIELD;
+            cap8 = f;
+        }
+    }
+    if (c->sys.size() > 1) {
+        bool table = true;
+        LaunchShape sh{};
+        sh.kernel = def.kernel;
+        sh.lanes = 8;
+        sh.walkers_per_block = 8;
+        sh.bits_in_smem = 1;
+        sh.thr_in_smem = 1;
+        for (auto &s : c->sys) table = table && smem_for(sh, s.p) <= (size_t)c->max_smem;
+        def.walkers_per_block = table ? 8 : 4;
+        return def;
+    }
+    auto waves = [&](long long cap) { return cap > 0 ? (need + cap - 1) / cap : (1ll << 40); };
+    const int cap16 = most(def.kernel, 16);
+    const bool g16 = waves(cap16) < waves(cap8);
+    const int cap = g16 ? cap16 : cap8, step = g16 ? 2 : 4;
+    const long long n = waves(cap), per = (need + n - 1) / n;
+    def.lanes_per_walker = g16 ? 16 : 8;
+    def.walkers_per_block = (int)std::min<long long>(cap, (per + step - 1) / step * step);
+    return def;
 }
 
 Context *as_ctx(void *p) { return static_cast<Context *>(p); }
@@ -780,17 +908,7 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
                                  "system %d: initial energy %d outside window [%d, %d]", i, v,
                                  s.desc.e_lo, s.desc.e_hi));
     }
-    // default launch: the field kernel when every system's fields fit in
-    // shared memory, else the group kernel with the bitsets in shared memory
-    // when they fit, else in global memory (8 lanes, 16 walkers per block)
-    mucal_launch_config def{MUCAL_KERNEL_FIELD, 8, 16, 1, 0, 1};
-    for (auto &s : c->sys)
-        if (smem_for(LaunchShape{MUCAL_KERNEL_FIELD, 8, 16, 1, 0, 0, 0}, s.p) > (size_t)c->max_smem)
-            def.kernel = MUCAL_KERNEL_GROUP;
-    if (def.kernel == MUCAL_KERNEL_GROUP)
-        for (auto &s : c->sys)
-            if (smem_for(LaunchShape{MUCAL_KERNEL_GROUP, 8, 16, 1, 0, 0, 0}, s.p) > (size_t)c->max_smem)
-                def.bits_in_smem = 0;
+    const mucal_launch_config def = default_launch(c);
     rc = apply_launch_config(c, def);
     if (rc != MUCAL_OK) return bail(rc);
     *out = c;
@@ -901,7 +1019,8 @@ int mucal_run_iteration(void *ctx, int64_t sweeps, uint32_t iteration)
                           a.walkers_per_block == b.walkers_per_block &&
                           a.bits_in_smem == b.bits_in_smem && a.thr_in_smem == b.thr_in_smem &&
                           a.smem_bytes == b.smem_bytes && a.persistent == b.persistent &&
-                          a.thr_window == b.thr_window && a.multi_commit == b.multi_commit;
+                          a.thr_window == b.thr_window && a.multi_commit == b.multi_commit &&
+                          a.scan_window == b.scan_window;
         if (!same) {
             int rc = capture_iteration(c, (uint64_t)sweeps, iteration, grid);
             if (rc != MUCAL_OK) return rc;
@@ -1168,6 +1287,7 @@ int mucal_set_tunnel_window(void *ctx, int32_t sys, int32_t e_min, int32_t e_max
     CUDA_TRY(c, cudaSetDevice(c->device));
     s.p.tun_lo = e_min - s.desc.e_lo;
     s.p.tun_hi = e_max - s.desc.e_lo;
+    for (auto &q : c->sys) q.p.tunnel = 1;
     rc = upload_sys_table(c);
     if (rc != MUCAL_OK) return rc;
     c->tunnel = true;

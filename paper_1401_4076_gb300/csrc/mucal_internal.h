@@ -29,8 +29,13 @@ struct SysParams {
     int32_t hist_rows;         // rows in use for the current launch shape
     const uint32_t *thr;       // [n_bins][tstride] acceptance thresholds (entries width..tstride-1
                                // of a row unused)
+    const uint32_t *thrT;      // dE-major copy of the table, [width][thrT_pitch]: the threshold of
+                               // bin b at thrT[j * thrT_pitch + kThrTPad + b], zeros around it
+                               // (NULL unless the launch shape's multi-commit rounds read it)
+    int32_t thrT_pitch;
     unsigned long long *accepts; // [n_walkers] accepted moves in the last iteration
     unsigned long long *H;     // [n_bins] summed histogram H(E) (Eq. 2)
+    int32_t tunnel;            // 1: keep the tunnelling books
     int32_t tun_lo, tun_hi;    // tunnelling ends as bins: a walker at bin <= tun_lo is at the
                                // low end, at bin >= tun_hi at the high end
     uint8_t *tun_state;        // [n_walkers] 0 = no end reached yet, 1 = low end last, 2 = high
@@ -38,6 +43,9 @@ struct SysParams {
     uint32_t *tun_count;       // [n_walkers] tunnelling events (end-to-end travels) so far
     unsigned int *err;         // set non-zero when a bounded wait of a walker kernel ran out
 };
+
+// Padding of the dE-major threshold rows on either side (words), a multiple of 4.
+constexpr int kThrTPad = 16;
 
 // Threshold-row window of the group and field kernels (threshold mode 2):
 // each walker keeps kThrWindowRows consecutive rows of the table in shared
@@ -59,8 +67,12 @@ struct BlockWork {
 // shared or global memory and the thresholds in global memory, in shared
 // memory or in a per-walker row window, and the field kernel with the three
 // threshold modes.
-constexpr int kWalkerUpdateFns = 4 + 5 * 2 * 3 + 5 * 3 + 4 * 6;   // last: multi-commit
-                                                                // kernels (NULL where absent)
+constexpr int kWalkerUpdateFns = 4 + 5 * 2 * 3 + 5 * 3;
+// Kernels of one lane count with several commits per round (persistent or
+// not, tunnelling bookkeeping or not): bitsets in shared memory, in global
+// memory or count fields, each with the thresholds in global memory, in
+// shared memory and in a row window per walker.
+constexpr int kWalkerScanFns = 9;
 
 struct LaunchShape {
     int kernel;             // MUCAL_KERNEL_THREAD / _GROUP / _FIELD
@@ -72,8 +84,9 @@ struct LaunchShape {
     int persistent;         // resident blocks pull work items from a counter
     int thr_window;         // (group and field kernels, when the table is not in shared
                             // memory) keep a window of rows per walker in shared memory
-    int multi_commit;       // (group and field kernels, 4+ lanes, no window, no tunnelling
-                            // bookkeeping) several commits per round
+    int multi_commit;       // (group and field kernels, 4+ lanes) several commits per round;
+                            // thr_window is then 0 and the next field tells
+    int scan_window;        // rounds with several commits on a window of rows per walker
 };
 
 // Kernel launchers (walker_kernels.cu).  All are asynchronous on `stream`.
@@ -105,6 +118,12 @@ const void *walker_update_fn_persist(const LaunchShape &shape);
 void walker_update_persist_fns(const void *(&fns)[kWalkerUpdateFns]);
 const void *walker_update_fn_persist_tun(const LaunchShape &shape);
 void walker_update_persist_tun_fns(const void *(&fns)[kWalkerUpdateFns]);
+// The kernels with several commits per round, one translation unit per lane
+// count (walker_scan_<lanes>.cu), in the order of kWalkerScanFns.
+void walker_scan_4_fns(const void *(&fns)[kWalkerScanFns]);
+void walker_scan_8_fns(const void *(&fns)[kWalkerScanFns]);
+void walker_scan_16_fns(const void *(&fns)[kWalkerScanFns]);
+void walker_scan_32_fns(const void *(&fns)[kWalkerScanFns]);
 // Shared-memory layout of a walker-update block: [threshold table][bitsets]
 // (group and thread kernels) or [threshold table][count fields] (field
 // kernel).
@@ -116,6 +135,8 @@ size_t field_smem_bytes(const SysParams &p);
 cudaError_t launch_hist_reduce(const SysParams *host_sys, const SysParams *dev_sys, int n_sys,
                                cudaStream_t stream);
 cudaError_t walker_update_max_smem(int *bytes);
+// Rewrite the dE-major copy of system p's threshold table from p.thr.
+cudaError_t launch_thr_transpose(const SysParams &p, cudaStream_t stream);
 
 // Replica exchange between neighbouring systems of a tempering ladder
 // (walker_kernels.cu): thr holds one row of `width` thresholds per pair.

@@ -96,6 +96,16 @@ __global__ void hist_reduce_kernel(SysParams p)
     if (sum) atomicAdd(p.H + b, sum);
 }
 
+// The dE-major copy of a threshold table: entry (b, j) to row j, word
+// kThrTPad + b.  Thread per entry of a row-padded table row.
+__global__ void thr_transpose_kernel(SysParams p, uint32_t *out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = i / p.tstride, j = i - b * p.tstride;
+    if (b < p.n_bins && j < p.width)
+        out[(size_t)j * p.thrT_pitch + kThrTPad + b] = p.thr[i];
+}
+
 // ---------------------------------------------------------------------------
 // Replica exchange (parallel tempering): systems k and k+1 (k = parity,
 // parity + 2, ...; blockIdx.y picks the pair) are copies of one lattice at
@@ -225,14 +235,21 @@ cudaError_t walker_update_max_smem(int *bytes)
     walker_update_tunnel_fns(fl[1]);
     walker_update_persist_fns(fl[2]);
     walker_update_persist_tun_fns(fl[3]);
-    const void *fns[4 * kWalkerUpdateFns];
-    for (int f = 0; f < 4; ++f)
-        for (int i = 0; i < kWalkerUpdateFns; ++i) fns[kWalkerUpdateFns * f + i] = fl[f][i];
+    const void *sc[4][kWalkerScanFns];
+    walker_scan_4_fns(sc[0]);
+    walker_scan_8_fns(sc[1]);
+    walker_scan_16_fns(sc[2]);
+    walker_scan_32_fns(sc[3]);
+    const void *fns[4 * (kWalkerUpdateFns + kWalkerScanFns)];
+    int n = 0;
+    for (int f = 0; f < 4; ++f) {
+        for (const void *fn : fl[f]) fns[n++] = fn;
+        for (const void *fn : sc[f]) fns[n++] = fn;
+    }
     // the dynamic limit leaves room for the largest static shared array (the
     // thread kernel's tunnelling words)
     size_t max_static = 0;
     for (const void *fn : fns) {
-        if (!fn) continue;   // flavour without a multi-commit kernel
         cudaFuncAttributes attr{};
         e = cudaFuncGetAttributes(&attr, fn);
         if (e != cudaSuccess) return e;
@@ -240,7 +257,6 @@ cudaError_t walker_update_max_smem(int *bytes)
     }
     *bytes -= (int)max_static;
     for (const void *fn : fns) {
-        if (!fn) continue;
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, *bytes);
         if (e != cudaSuccess) return e;
     }
@@ -249,6 +265,18 @@ cudaError_t walker_update_max_smem(int *bytes)
 
 const void *walker_update_fn(const LaunchShape &shape, bool tunnel)
 {
+    if (shape.multi_commit) {      // (4 lanes or more)
+        const void *fns[kWalkerScanFns];
+        switch (shape.lanes) {
+        case 4: walker_scan_4_fns(fns); break;
+        case 8: walker_scan_8_fns(fns); break;
+        case 16: walker_scan_16_fns(fns); break;
+        case 32: walker_scan_32_fns(fns); break;
+        default: return nullptr;
+        }
+        const int view = shape.kernel == 2 ? 2 : (shape.bits_in_smem ? 0 : 1);
+        return fns[3 * view + (shape.thr_in_smem ? 1 : (shape.scan_window ? 2 : 0))];
+    }
     if (shape.persistent)
         return tunnel ? walker_update_fn_persist_tun(shape) : walker_update_fn_persist(shape);
     return tunnel ? walker_update_fn_tunnel(shape) : walker_update_fn_t<false, false>(shape);
@@ -285,6 +313,13 @@ cudaError_t launch_walker_update(const SysParams *dev_sys, const BlockWork *dev_
                     (void *)&n_items, (void *)&counter};
     return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)(shape.walkers_per_block * shape.lanes)),
                             args, shape.smem_bytes, stream);
+}
+
+cudaError_t launch_thr_transpose(const SysParams &p, cudaStream_t stream)
+{
+    const int total = p.n_bins * p.tstride;
+    thr_transpose_kernel<<<(total + 255) / 256, 256, 0, stream>>>(p, const_cast<uint32_t *>(p.thrT));
+    return cudaGetLastError();
 }
 
 size_t thr_smem_words(const SysParams &p) { return thr_words_aligned(p); }
