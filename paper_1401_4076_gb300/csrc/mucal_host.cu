@@ -23,6 +23,9 @@ namespace {
 
 thread_local std::string g_init_error;
 
+// Lists of all walkers up to this size stay in L2 (129 MB) by themselves.
+constexpr size_t kListsInL2 = (size_t)64 << 20;
+
 struct System {
     mucal_system_desc desc{};
     SysParams p{};                  // host copy holding device pointers
@@ -501,98 +504,124 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
     return MUCAL_OK;
 }
 
-// The launch shape of a new context: several commits per round, 8 lanes per
-// walker, on count fields or on the bitsets.
+// Lanes per walker (the window of attempts a round decides) for r walkers
+// beside each other on an SM and N particles.
+//
+// Two attempts of a window touch with a chance of about 3 / N, which bounds
+// the useful window; below that, few walkers leave issue slots for wider
+// windows, many need narrow ones, whose instructions per attempt are fewer.
+// Measured on GB300 (ms of the walker update at 4 / 8 / 16 / 32 lanes): 3D
+// L = 33, N = 3244, r = 1: 8.86 / 5.06 / 3.37 / 2.85; 3D L = 24, N = 1382,
+// r = 14: 7.75 / 4.51 / 3.82 / 6.9; 3D L = 32, N = 3277, r = 28: 18.3 / 12.4 /
+// 13.0 / -; 2D L = 64, N = 410, r = 1: 4.29 / 2.74 / 2.28 / 2.79, r = 10: 4.35 /
+// 2.80 / 3.05 / 7.3; 3D L = 8, N = 56, r = 56: 1.44 / 1.98 / 5.2 / -; 2D
+// L = 14, N = 17, r = 19: 0.51 / 0.65 / 1.40 / -.
+int default_lanes(long long r, double N)
+{
+    if (N < 32 || (N < 200 && r > 40)) return 4;
+    if (N >= 2500 && r <= 7) return 32;
+    if ((N >= 1000 && r <= 24) || (N >= 300 && r <= 4)) return 16;
+    return 8;
+}
+
+// The launch shape of a new context: several commits per round.
 //
 // A walker is a serial chain, so what counts is that all walkers run at once,
 // or in equal waves, with as many of them beside each other on an SM as its
 // shared memory holds.  One system: its walkers per SM are split into the
-// fewest waves that fit, one block per SM and wave.  Measured on GB300 (ms of
-// the walker update, 16 walkers per block against this rule): 2D L = 64,
-// N = 410, 4096 walkers, 50 sweeps 3.75 -> 3.11 (28 walkers, one wave); 3D
-// L = 32, N = 3277, 8192 walkers, 10 sweeps 13.4 -> 12.8 (28, two waves); 2D
-// L = 74, N = 100, 1024 walkers, 137 sweeps 1.81 -> 1.77 (8, one wave).  Where
-// blocks of 4, 8, 12... walkers at 8 lanes need a wave more than blocks of
-// 2, 4, 6... at 16 lanes, 16 lanes: 3D L = 48, N = 11059, 2048 walkers,
-// 4 sweeps 14.1 (12 walkers, two waves) -> 6.7 (14, one wave).  Several
-// systems: small blocks, which pack their uneven bitsets and lengths best
-// (the 27-system batch, 5 sweeps: 8 walkers 12.4, 4 walkers 10.8).
+// fewest waves that fit, one block per SM and wave.  Measured (blocks of 16
+// walkers against this rule): 2D L = 64, N = 410, 4096 walkers, 20 sweeps
+// 1.24 -> 1.17 ms (28 walkers, one wave); 3D L = 32, N = 3277, 8192 walkers, 10
+// sweeps 15.9 -> 12.4 (28, two waves).  Several systems: small blocks, which
+// pack their uneven bitsets and lengths best (the 27-system batch, 5 sweeps:
+// 4 walkers 9.2, 14 walkers 10.9), of 8 walkers where a block stages the
+// table.
 //
-// Fields (two byte loads per attempt instead of 4d words, 4d more atomics per
-// commit) where they fit 16 walkers to a block and do not cost a resident
-// walker: 2D L = 64 3.24 (bitsets) -> 3.11, but five 2D systems of L = 61 to
-// 97, 5120 walkers, 50 sweeps 1.10 (bitsets) against 1.95.
+// Count fields (two byte loads per attempt instead of 4d words, 4d more
+// atomics per commit) where they fit 16 walkers to a block and do not cost a
+// resident walker: 2D L = 64 3.24 (bitsets) -> 3.11, but five 2D systems of
+// L = 61 to 97, 5120 walkers, 50 sweeps 1.06 (bitsets) against 1.9.
+//
+// Below 16 particles nearly every window holds a conflict, and the rounds with
+// one commit are as fast or faster: 2D L = 22, N = 12, 64 walkers 0.122 against
+// 0.122 ms at acceptance 0.5, 0.089 against 0.116 at 0.1.
 mucal_launch_config default_launch(Context *c)
 {
     long long total = 0;
-    for (auto &s : c->sys) total += s.p.n_walkers;
+    double work = 0.0, work_n = 0.0;
+    for (auto &s : c->sys) {
+        total += s.p.n_walkers;
+        work += (double)s.p.n_walkers * s.p.N;
+        work_n += (double)s.p.n_walkers * s.p.N * s.p.N;
+    }
+    const double N = work_n / work;     // particles of the system an average attempt belongs to
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     const long long need = (total + sms - 1) / sms;     // walkers per SM
-    auto fits = [&](int kernel, int lanes, int w, int bits) {
-        LaunchShape sh{};
-        sh.kernel = kernel;
-        sh.lanes = lanes;
-        sh.walkers_per_block = w;
-        sh.bits_in_smem = bits;
-        sh.thr_in_smem = 1;
-        bool table = true, window = true;
-        for (auto &s : c->sys) table = table && smem_for(sh, s.p) <= (size_t)c->max_smem;
-        if (table) return true;
-        sh.thr_in_smem = 0;
-        sh.scan_window = 1;
-        for (auto &s : c->sys) window = window && smem_for(sh, s.p) <= (size_t)c->max_smem;
-        return window;
+    // whether w walkers fit a block: 0 no, 1 with row windows, 2 with the table
+    auto fits = [&](int kernel, int w) {
+        for (int table = 1; table >= 0; --table) {
+            LaunchShape sh{};
+            sh.kernel = kernel;
+            sh.walkers_per_block = w;
+            sh.bits_in_smem = 1;
+            sh.thr_in_smem = table;
+            sh.scan_window = 1;
+            bool ok = true;
+            for (auto &s : c->sys) ok = ok && smem_for(sh, s.p) <= (size_t)c->max_smem;
+            if (ok) return 1 + table;
+        }
+        return 0;
     };
-    auto plain_fits = [&](int kernel) {
-        bool ok = true;
+    auto plain_fits = [&](int kernel) {      // without table and windows
         LaunchShape sh{};
         sh.kernel = kernel;
-        sh.lanes = 8;
         sh.walkers_per_block = 16;
         sh.bits_in_smem = 1;
+        bool ok = true;
         for (auto &s : c->sys) ok = ok && smem_for(sh, s.p) <= (size_t)c->max_smem;
         return ok;
     };
-    mucal_launch_config def{MUCAL_KERNEL_GROUP, 8, 16, 1, 0, 0, 1};
-    if (!plain_fits(MUCAL_KERNEL_GROUP) && !fits(MUCAL_KERNEL_GROUP, 8, 4, 1)) {
-        def.bits_in_smem = 0;
-        return def;
-    }
-    // the most walkers a block can hold (an SM's, at one block per SM)
-    auto most = [&](int kernel, int lanes) {
-        const int step = 32 / lanes;
+    auto most = [&](int kernel) {            // walkers an SM's shared memory holds
         int w = 0;
-        while ((w + step) * lanes <= 512 && fits(kernel, lanes, w + step, 1)) w += step;
+        while (w < 128 && fits(kernel, w + 1)) ++w;
         return w;
     };
-    int cap8 = most(MUCAL_KERNEL_GROUP, 8);
-    if (plain_fits(MUCAL_KERNEL_FIELD)) {
-        const int f = most(MUCAL_KERNEL_FIELD, 8);
-        if (f >= need || f >= cap8) {
-            def.kernel = MUCAL_KERNEL_FIELD;
-            cap8 = f;
-        }
-    }
-    if (c->sys.size() > 1) {
-        bool table = true;
-        LaunchShape sh{};
-        sh.kernel = def.kernel;
-        sh.lanes = 8;
-        sh.walkers_per_block = 8;
-        sh.bits_in_smem = 1;
-        sh.thr_in_smem = 1;
-        for (auto &s : c->sys) table = table && smem_for(sh, s.p) <= (size_t)c->max_smem;
-        def.walkers_per_block = table ? 8 : 4;
+    mucal_launch_config def{MUCAL_KERNEL_GROUP, 8, 16, 1, 0, 0, 1};
+    long long cap = most(MUCAL_KERNEL_GROUP);
+    if (cap < 1) {                           // bitsets in global memory
+        def.bits_in_smem = 0;
+        def.lanes_per_walker = default_lanes(need, N);
+        if (def.lanes_per_walker == 4) def.lanes_per_walker = 8;
         return def;
     }
-    auto waves = [&](long long cap) { return cap > 0 ? (need + cap - 1) / cap : (1ll << 40); };
-    const int cap16 = most(def.kernel, 16);
-    const bool g16 = waves(cap16) < waves(cap8);
-    const int cap = g16 ? cap16 : cap8, step = g16 ? 2 : 4;
-    const long long n = waves(cap), per = (need + n - 1) / n;
-    def.lanes_per_walker = g16 ? 16 : 8;
-    def.walkers_per_block = (int)std::min<long long>(cap, (per + step - 1) / step * step);
+    if (plain_fits(MUCAL_KERNEL_FIELD)) {
+        const int f = most(MUCAL_KERNEL_FIELD);
+        if (f >= need || f >= cap) {
+            def.kernel = MUCAL_KERNEL_FIELD;
+            cap = f;
+        }
+    }
+    if (N < 16) {
+        def.multi_commit = 0;
+        def.thr_window = 1;
+        if (!plain_fits(def.kernel)) def.bits_in_smem = 0;
+        return def;
+    }
+    const bool one = c->sys.size() == 1;
+    const long long waves = (need + cap - 1) / cap;
+    const long long r = one ? (need + waves - 1) / waves : std::min(need, cap);
+    const long long want = one ? r : (fits(def.kernel, 8) == 2 ? 8 : 4);
+    // whole warps: blocks of 32 / lanes walkers and multiples; wider groups
+    // come in finer blocks
+    for (int lanes = default_lanes(r, N);; lanes *= 2) {
+        const long long step = 32 / lanes;
+        const long long top = std::min<long long>(cap, 512 / lanes) / step * step;
+        const long long w = (want + step - 1) / step * step;
+        def.lanes_per_walker = lanes;
+        def.walkers_per_block = (int)std::min(w, top);
+        if (top >= step && (w <= top || lanes >= 16)) break;    // (at 32 lanes always)
+    }
     return def;
 }
 
@@ -870,6 +899,9 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
             cudaMemsetAsync(p.tun_count, 0, nw * 4, c->stream) != cudaSuccess)
             return bail(fail(nullptr, MUCAL_ERR_CUDA, "memset failed"));
     }
+    size_t lists = 0;
+    for (auto &s : c->sys) lists += (size_t)s.p.n_walkers * (size_t)s.p.V * (s.p.idx16 ? 2 : 4);
+    for (auto &s : c->sys) s.p.prefetch = lists > kListsInL2 ? 1 : 0;
     if (cudaMalloc(&c->d_next_item, sizeof(int)) != cudaSuccess)
         return bail(fail(nullptr, MUCAL_ERR_OOM, "cudaMalloc of the work-item counter failed"));
     if (cudaMalloc(&c->d_walk_err, sizeof(unsigned int)) != cudaSuccess ||

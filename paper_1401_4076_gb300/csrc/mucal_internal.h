@@ -35,6 +35,7 @@ struct SysParams {
     int32_t thrT_pitch;
     unsigned long long *accepts; // [n_walkers] accepted moves in the last iteration
     unsigned long long *H;     // [n_bins] summed histogram H(E) (Eq. 2)
+    int32_t prefetch;          // 1: the context's lists are larger than L2
     int32_t tunnel;            // 1: keep the tunnelling books
     int32_t tun_lo, tun_hi;    // tunnelling ends as bins: a walker at bin <= tun_lo is at the
                                // low end, at bin >= tun_hi at the high end

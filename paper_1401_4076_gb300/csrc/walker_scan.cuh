@@ -10,40 +10,53 @@ namespace mucal {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Several commits per round (multi-commit rounds) on a sliding window of G
-// attempts: lane t mod G of the group holds attempt t, for the G attempts from
-// the first undecided one (t0) on.
+// Several commits per round (multi-commit rounds) on a sliding window of W
+// attempts, one per lane of the walker's group: slot (lane) t mod W holds
+// attempt t, for the W attempts from the first undecided one (t0) on.  The
+// place of a slot is its distance from t0's slot.
 //
 // A round evaluates the energy changes of the whole window against the state
 // at its start.  Such a value stays right until an earlier attempt of the
-// window commits a move next to one of the lane's two sites or in one of its
-// two list slots; which earlier lanes could do so (cm, a bit mask) is a matter
-// of the sites alone.  Taking all energy changes as they are, the decisions
-// are a short serial recurrence in the energy, which every lane of the group
-// runs redundantly in registers: T(E, dE_i) >= r_i ? E += dE_i.  The round
-// then ends at the first lane whose cm meets an accepted lane: the lanes
-// before it are decided as the serial chain decides them, commit together and
-// take the next attempts, and the window slides on.  The first lane is never
-// stopped, so every round decides at least one attempt, mostly the whole
-// window; no group of a warp waits for another's conflicts.
+// window commits a move next to one of the attempt's two sites or in one of
+// its two list slots; which attempts touch which is a matter of the sites
+// alone.  Taking all energy changes as they are, the decisions are a short
+// serial recurrence in the energy, which every lane of the group runs
+// redundantly in registers: T(E, dE_i) >= r_i ? E += dE_i.  The round then
+// ends at the first attempt that an earlier accepted one touches: the
+// attempts before it are decided as the serial chain decides them, commit
+// together and give way to the next ones, and the window slides on.  The first
+// attempt is never stopped, so every round decides at least one, mostly the
+// whole window; no group of a warp waits for another's conflicts.
+//
+// The rounds are bound by the latency of dependent integer instructions and by
+// issue slots (a walker is one serial chain, and an SM holds only tens of
+// walkers): on 2D L = 64 at 8 lanes and 28 walkers per SM a round is about 540
+// warp instructions, one issued every 4.0 cycles per warp, for 7.3 attempts
+// per walker (18.3 warp instructions per attempt against 24 with one commit
+// per round; 2.9e10 against 1.7e10 attempts/s).  So independent work stands
+// beside the recurrence, in the same straight line of code: the random
+// numbers (2.77e10 -> 2.86e10 attempts/s) and the comparisons of the moves'
+// sites (-> 2.95e10).  Two attempts per lane, which halve what is done once
+// per lane, issued as much and ran at half the warps: 2.07e10.
 //
 // A step of the recurrence is one threshold load from shared memory and a few
 // dependent integer instructions: from the whole table (kThrShared), or from
-// the walker's window of rows (kThrWindow, see ThrWindow), where a lane
+// the walker's window of rows (kThrWindow, see ThrWindow), where an attempt
 // reached with an energy whose row has not arrived is stopped like one with a
 // conflict.  Where neither fits, the thresholds are read from global memory
 // (kThrGlobal) ahead of the recurrence: every lane turns the kScanWords
-// thresholds of its dE around the round's energy, contiguous in the table's
-// dE-major copy, into a bit mask of decisions by energy, and is stopped when
-// reached with another energy.
+// thresholds of an attempt's dE around the round's energy, contiguous in the
+// table's dE-major copy, into a bit mask of decisions by energy, and the
+// attempt is stopped when reached with another energy.
 // ---------------------------------------------------------------------------
 constexpr int kScanWords = 24;    // energies of a decision mask (bits 0-23; the lane's dE above)
+constexpr int kScanFew = 2;       // accepted moves of a walker's round that are still few
 constexpr int kScanDrift = 5;     // a window's centre follows an energy further from it than this
 constexpr int kScanReach = 10;    // of which at least this many on either side of the round's energy
 static_assert(kThrTPad >= kScanReach + 3 && kThrTPad >= kScanWords - kScanReach, "window in the padding");
 
-// Occupation as the rounds read it: d4() is 4 times the energy change but for
-// the adjacency of the two sites, commit() applies this lane's move (several
+// Occupation as the rounds read it: de() is the energy change but for the
+// adjacency of the two sites, commit() applies this lane's move (several
 // lanes of a group may commit at once, so through atomics).
 template <int D, bool SB>
 struct ScanBits {
@@ -59,13 +72,13 @@ struct ScanBits {
         }
         return (v >> (s & 31u)) & 1u;
     }
-    __device__ __forceinline__ int d4(uint32_t, uint32_t, const uint32_t (&na)[2 * D],
+    __device__ __forceinline__ int de(uint32_t, uint32_t, const uint32_t (&na)[2 * D],
                                       const uint32_t (&nb)[2 * D]) const
     {
         int n = 0;
 #pragma unroll
         for (int i = 0; i < 2 * D; ++i) n += (int)bit(na[i]) - (int)bit(nb[i]);
-        return 4 * n;
+        return n;
     }
     __device__ __forceinline__ void commit(uint32_t a, uint32_t b, const uint32_t (&)[2 * D],
                                            const uint32_t (&)[2 * D]) const
@@ -78,13 +91,13 @@ struct ScanBits {
 template <int D>
 struct ScanField {
     uint32_t fbase;      // shared byte address of the walker's field (see FieldView)
-    __device__ __forceinline__ int d4(uint32_t a, uint32_t b, const uint32_t (&)[2 * D],
+    __device__ __forceinline__ int de(uint32_t a, uint32_t b, const uint32_t (&)[2 * D],
                                       const uint32_t (&)[2 * D]) const
     {
         uint32_t va, vb;
         asm volatile("ld.shared.u8 %0, [%1];" : "=r"(va) : "r"(fbase + a) : "memory");
         asm volatile("ld.shared.u8 %0, [%1];" : "=r"(vb) : "r"(fbase + b) : "memory");
-        return (int)va - (int)vb;
+        return ((int)va - (int)vb) >> 2;
     }
     __device__ __forceinline__ void commit(uint32_t, uint32_t, const uint32_t (&na)[2 * D],
                                            const uint32_t (&nb)[2 * D]) const
@@ -107,21 +120,98 @@ struct Sizes {
     uint32_t magL;
 };
 
-template <int D, typename IdxT, int G, int TM, typename View>
+// The round's comparisons as chains of predicates, one instruction each (the
+// compiled form of the same C++ expressions materialised every comparison as a
+// number: 505 against 270 comparing and selecting instructions a round in 2D).
+
+// set |= bit if one of the sites s is x or y, or pa == a or pb == b.
+template <int D>
+__device__ __forceinline__ void or_if_touch(uint32_t &set, uint32_t bit, const uint32_t (&na)[2 * D],
+                                            const uint32_t (&nb)[2 * D], uint32_t a, uint32_t b,
+                                            uint32_t pa, uint32_t pb)
+{
+    if constexpr (D == 2)
+        asm("{\n\t.reg .pred p, q;\n\t"
+            "setp.eq.u32 p, %10, %12;\n\tsetp.eq.u32 q, %11, %13;\n\t"
+            "setp.eq.or.u32 p, %2, %12, p;\n\tsetp.eq.or.u32 q, %2, %13, q;\n\t"
+            "setp.eq.or.u32 p, %3, %12, p;\n\tsetp.eq.or.u32 q, %3, %13, q;\n\t"
+            "setp.eq.or.u32 p, %4, %12, p;\n\tsetp.eq.or.u32 q, %4, %13, q;\n\t"
+            "setp.eq.or.u32 p, %5, %12, p;\n\tsetp.eq.or.u32 q, %5, %13, q;\n\t"
+            "setp.eq.or.u32 p, %6, %12, p;\n\tsetp.eq.or.u32 q, %6, %13, q;\n\t"
+            "setp.eq.or.u32 p, %7, %12, p;\n\tsetp.eq.or.u32 q, %7, %13, q;\n\t"
+            "setp.eq.or.u32 p, %8, %12, p;\n\tsetp.eq.or.u32 q, %8, %13, q;\n\t"
+            "setp.eq.or.u32 p, %9, %12, p;\n\tsetp.eq.or.u32 q, %9, %13, q;\n\t"
+            "@p or.b32 %0, %0, %1;\n\t@q or.b32 %0, %0, %1;\n\t}"
+            : "+r"(set)
+            : "r"(bit), "r"(na[0]), "r"(na[1]), "r"(na[2]), "r"(na[3]), "r"(nb[0]), "r"(nb[1]),
+              "r"(nb[2]), "r"(nb[3]), "r"(a), "r"(b), "r"(pa), "r"(pb));
+    else
+        asm("{\n\t.reg .pred p, q;\n\t"
+            "setp.eq.u32 p, %14, %16;\n\tsetp.eq.u32 q, %15, %17;\n\t"
+            "setp.eq.or.u32 p, %2, %16, p;\n\tsetp.eq.or.u32 q, %2, %17, q;\n\t"
+            "setp.eq.or.u32 p, %3, %16, p;\n\tsetp.eq.or.u32 q, %3, %17, q;\n\t"
+            "setp.eq.or.u32 p, %4, %16, p;\n\tsetp.eq.or.u32 q, %4, %17, q;\n\t"
+            "setp.eq.or.u32 p, %5, %16, p;\n\tsetp.eq.or.u32 q, %5, %17, q;\n\t"
+            "setp.eq.or.u32 p, %6, %16, p;\n\tsetp.eq.or.u32 q, %6, %17, q;\n\t"
+            "setp.eq.or.u32 p, %7, %16, p;\n\tsetp.eq.or.u32 q, %7, %17, q;\n\t"
+            "setp.eq.or.u32 p, %8, %16, p;\n\tsetp.eq.or.u32 q, %8, %17, q;\n\t"
+            "setp.eq.or.u32 p, %9, %16, p;\n\tsetp.eq.or.u32 q, %9, %17, q;\n\t"
+            "setp.eq.or.u32 p, %10, %16, p;\n\tsetp.eq.or.u32 q, %10, %17, q;\n\t"
+            "setp.eq.or.u32 p, %11, %16, p;\n\tsetp.eq.or.u32 q, %11, %17, q;\n\t"
+            "setp.eq.or.u32 p, %12, %16, p;\n\tsetp.eq.or.u32 q, %12, %17, q;\n\t"
+            "setp.eq.or.u32 p, %13, %16, p;\n\tsetp.eq.or.u32 q, %13, %17, q;\n\t"
+            "@p or.b32 %0, %0, %1;\n\t@q or.b32 %0, %0, %1;\n\t}"
+            : "+r"(set)
+            : "r"(bit), "r"(na[0]), "r"(na[1]), "r"(na[2]), "r"(na[3]), "r"(na[4]), "r"(na[5]),
+              "r"(nb[0]), "r"(nb[1]), "r"(nb[2]), "r"(nb[3]), "r"(nb[4]), "r"(nb[5]), "r"(a), "r"(b),
+              "r"(pa), "r"(pb));
+}
+
+// x += v if y == z.
+__device__ __forceinline__ void add_if_eq(uint32_t &x, uint32_t v, uint32_t y, uint32_t z)
+{
+    asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, %3;\n\t@p add.u32 %0, %0, %1;\n\t}"
+        : "+r"(x) : "r"(v), "r"(y), "r"(z));
+}
+
+// A step of the recurrence: if T >= r, x += v and set |= bit.
+__device__ __forceinline__ void step_if_ge(int &x, int v, unsigned &set, unsigned bit, uint32_t T, uint32_t r)
+{
+    asm("{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %4, %5;\n\t@p add.s32 %0, %0, %2;\n\t"
+        "@p or.b32 %1, %1, %3;\n\t}"
+        : "+r"(x), "+r"(set) : "r"(v), "r"(bit), "r"(T), "r"(r));
+}
+
+// Bits of x turned left by n places in W bits (n <= W).
+template <int W>
+__device__ __forceinline__ unsigned turn_left(unsigned x, uint32_t n)
+{
+    if constexpr (W == 32) return __funnelshift_l(x, x, n);
+    else return ((x << n) | ((x << n) >> W)) & ((1u << W) - 1u);
+}
+
+template <int D, typename IdxT, int W, int TM, typename View>
 __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool active, const View v,
                                            const uint32_t *thr, unsigned long long *hist,
-                                           uint64_t A, uint32_t iter, uint32_t ring_s, uint32_t mbar_s)
+                                           uint64_t A, uint32_t iter, uint32_t ring_s, uint32_t mbar_s,
+                                           uint32_t *stage_all)
 {
     constexpr unsigned FULL = 0xffffffffu;
-    constexpr unsigned GMASK = (G == 32) ? 0xffffffffu : ((1u << G) - 1u);
+    constexpr unsigned WM = (uint32_t)(W - 1);
     constexpr int NS = 2 * D;
     constexpr int TS = (4 * D + 1 + 3) & ~3;   // words of a table row (SysParams::tstride)
-    // an entry of a row's padding, where T = 0: what lanes without a decision to take read
-    constexpr uint32_t DEAD = 4u * (2 * D + 1);
+    constexpr bool PAIR = sizeof(IdxT) == 2;   // two list values fit one word
+    // dE + 2D of an attempt; one past the last, a row's padding, where T = 0,
+    // stands for an attempt past the end
+    constexpr uint32_t DEAD = 4 * D + 1;
+    constexpr unsigned GMASK = W == 32 ? 0xffffffffu : ((1u << W) - 1u);
     const int lane = threadIdx.x & 31;
-    const int j = lane & (G - 1);
+    const int j = lane & (W - 1);
     const int gbase = lane - j;
     const unsigned gm = GMASK << gbase;
+    // the group's words of shared memory, one per slot: used in turns, with a
+    // warp barrier before each write and after it
+    uint32_t *stage = stage_all + (threadIdx.x / W) * W;
     IdxT *S = walker_S<IdxT>(p, w);
     const uint32_t N = (uint32_t)p.N;
     const uint32_t holes = (uint32_t)(p.V - p.N);
@@ -129,8 +219,9 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     const Sizes sz{p.L, p.V, p.L2, p.magL};
     const uint32_t pitch = (uint32_t)p.thrT_pitch;
+    const bool ahead = p.prefetch != 0;
     int bin = active ? p.E[w] - p.e_lo : 0;
-    const uint32_t rbase = TM == kThrShared ? (uint32_t)__cvta_generic_to_shared(thr) + 8u * D : 0u;
+    const uint32_t rbase = TM == kThrShared ? (uint32_t)__cvta_generic_to_shared(thr) : ring_s;
     uint32_t carry = 0;      // attempts of the run at the current energy not recorded yet
     uint32_t acc = 0;
     // tunnelling bookkeeping (Sec. 4): every energy the walker takes is
@@ -165,15 +256,10 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
         vlo = bin - WLO;
         vhi = bin + WHI;
     }
-    // lane masks of a group turned so that bit o is the window's o-th attempt
-    auto turned = [](unsigned x, uint32_t h) -> unsigned {
-        if constexpr (G == 32) return __funnelshift_r(x, x, h);
-        else return ((x | (x << G)) >> h) & GMASK;
-    };
-    // attempt t0 + pos of this lane: the current one (k, m, a, b, r2p), the
-    // lane's next (n: attempt + G; its list entries are read in every round)
-    // and the one after it (q: its random numbers are drawn in every round,
-    // and its list entries prefetched into L2)
+    // the slot's attempt t: the current one (k, m, a, b, r2p), its next
+    // (n: attempt t + W; its list entries are read in every round) and the one
+    // after it (q: its random numbers are drawn in every round, and its list
+    // entries prefetched into L2 where the lists are larger than L2)
     auto draw = [&](uint64_t t, uint32_t &kk, uint32_t &mm, uint32_t &rr) {
         const uint4 r = philox10(make_uint4((uint32_t)t, (uint32_t)(t >> 32), iter, 0u), k0, k1);
         kk = __umulhi(r.x, N);
@@ -182,15 +268,140 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
         rr = (r.z == 0xFFFFFFFFu) ? r.z : r.z + 1u;
     };
     uint64_t t0 = 0;             // (the same in the whole group)
-    uint32_t k, m, r2p, kn, mn, r2n;
-    draw((uint64_t)j, k, m, r2p);
-    draw((uint64_t)j + G, kn, mn, r2n);
-    uint32_t a = 0, b = 1;       // any two sites, where there is no attempt
-    if (active && (uint64_t)j < A) {
+    uint32_t k, m, r2p, kn, mn, r2n, a, b;
+    const uint64_t t = (uint64_t)j;
+    draw(t, k, m, r2p);
+    draw(t + W, kn, mn, r2n);
+    a = 0;                       // any two sites, where there is no attempt
+    b = 1;
+    if (active && t < A) {
         a = __ldcg(S + k);
         b = __ldcg(S + N + m);
     }
+    // A round's values: attempts left, as far as the window and the next two
+    // windows reach; the place of t0's slot and of this one; the slot's next
+    // list entries and the random numbers of the attempt after; the sites
+    // around its move and dE + 2D.
+    uint32_t near, h, place, an, bn, kq, mq, r2q, code;
+    uint32_t na[NS], nb[NS];
+    unsigned am;              // accepted attempts, by place
+    int x0 = 0;
+    int xs[W];                // the energy bin after each attempt
+    auto begin = [&]() {
+        const uint64_t left = active && t0 < A ? A - t0 : 0u;
+        near = left < 3u * W ? (uint32_t)left : 3u * W;
+        h = (uint32_t)t0 & WM;
+        place = ((uint32_t)j - h) & WM;
+        an = a;
+        bn = b;
+        if (place + W < near) {
+            an = __ldcg(S + kn);
+            bn = __ldcg(S + N + mn);
+        }
+        neighbours<D>(sz, a, na);
+        neighbours<D>(sz, b, nb);
+        uint32_t de = (uint32_t)(v.de(a, b, na, nb) + 2 * D);
+#pragma unroll
+        for (int i = 0; i < NS; ++i) add_if_eq(de, 1u, na[i], b);    // (at most one of them)
+        code = place < near ? de : DEAD;
+    };
+    // The recurrence, and beside it, since its steps wait for one another,
+    // the slots' random numbers two windows ahead.
+    auto recurrence = [&]() {
+        am = 0;
+        draw(t0 + place + 2 * W, kq, mq, r2q);
+        if constexpr (TM != kThrGlobal) {
+            uint32_t rs[W], cs[W / 4];
+            __syncwarp(FULL);
+            stage[place] = r2p;
+            __syncwarp(FULL);
+#pragma unroll
+            for (int i = 0; i < W; i += 4) *reinterpret_cast<uint4 *>(rs + i) = *reinterpret_cast<const uint4 *>(stage + i);
+            __syncwarp(FULL);
+            reinterpret_cast<uint8_t *>(stage)[place] = (uint8_t)code;
+            __syncwarp(FULL);
+#pragma unroll
+            for (int i = 0; i < W / 4; ++i) cs[i] = stage[i];
+            int x = bin;
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                const uint32_t ci = (cs[i / 4] >> (8 * (i & 3))) & 0xFFu;
+                const uint32_t row = TM == kThrWindow ? (uint32_t)x & (kThrWindowRows - 1u) : (uint32_t)x;
+                uint32_t T;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(T) : "r"(row * (4u * TS) + (rbase + 4u * ci)));
+                step_if_ge(x, (int)ci - 2 * D, am, 1u << i, T, rs[i]);
+                xs[i] = x;
+            }
+        } else {
+            const int e0 = (bin + kThrTPad - kScanReach) & ~3;
+            x0 = bin + kThrTPad - e0;
+            uint32_t word;
+            const bool valid = place < near;
+            const uint4 *q = reinterpret_cast<const uint4 *>(
+                thr + ((valid ? code : 0u) * pitch + (uint32_t)e0));
+            uint32_t ok = 0;
+#pragma unroll
+            for (int g = 0; g < kScanWords / 4; ++g) {
+                const uint4 y = __ldg(q + g);
+                ok |= (y.x >= r2p ? 1u << (4 * g) : 0u) | (y.y >= r2p ? 2u << (4 * g) : 0u) |
+                      (y.z >= r2p ? 4u << (4 * g) : 0u) | (y.w >= r2p ? 8u << (4 * g) : 0u);
+            }
+            word = (code << 24) | (valid ? ok : 0u);
+            uint32_t ws[W];
+            __syncwarp(FULL);
+            stage[place] = word;
+            __syncwarp(FULL);
+#pragma unroll
+            for (int i = 0; i < W; i += 4) *reinterpret_cast<uint4 *>(ws + i) = *reinterpret_cast<const uint4 *>(stage + i);
+            int x = x0;
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                step_if_ge(x, (int)(ws[i] >> 24) - 2 * D, am, 1u << i,
+                           __funnelshift_r(ws[i], ws[i], (uint32_t)x) & 1u, 1u);
+                xs[i] = bin + x - x0;
+            }
+        }
+    };
+    // the window's places that hold an attempt
+    auto places = [&]() {
+        return W == 32 && near >= 32u ? 0xffffffffu : (1u << (near < W ? near : W)) - 1u;
+    };
+    auto prefetch = [&]() {
+        if (ahead && place + 2 * W < near) {
+            asm volatile("prefetch.L2 [%0];" ::"l"(S + kq));
+            asm volatile("prefetch.L2 [%0];" ::"l"(S + N + mq));
+        }
+    };
+    // what the slot goes on with: its next attempt, or the same one again
+    auto advance = [&](bool decided) {
+        k = decided ? kn : k;
+        m = decided ? mn : m;
+        a = decided ? an : a;
+        b = decided ? bn : b;
+        r2p = decided ? r2n : r2p;
+        kn = decided ? kq : kn;
+        mn = decided ? mq : mn;
+        r2n = decided ? r2q : r2n;
+    };
+    bool many = true;            // (the same in the whole warp) how the last round went:
+    bool quiet = false;          // many accepted moves, or none in the whole warp
     while (__any_sync(FULL, active && t0 < A)) {
+        // As long as no walker of the warp moves there is nothing to try for
+        // conflicts, commit or patch: rounds of the recurrence alone (a round
+        // that meets an accepted move is begun again below).
+        while (quiet) {
+            begin();
+            recurrence();
+            prefetch();
+            if (__any_sync(FULL, (am & places()) != 0u)) break;
+            const uint32_t nd = near < W ? near : (uint32_t)W;
+            advance(place < nd);
+            carry += nd;
+            t0 += nd;
+            const bool more = __any_sync(FULL, active && t0 < A);
+            const bool full = __any_sync(FULL, carry >= 0x40000000u);   // (recorded below)
+            quiet = more && !full;
+        }
         if constexpr (TM == kThrWindow) {
             // rows asked for a round ago; then the window follows the energy
             if (active && t0 < A) {
@@ -215,136 +426,115 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
                 if (tw.broken) t0 = A;     // the walker stops; the host reports the iteration invalid
             }
         }
-        const uint32_t h = (uint32_t)t0 & (uint32_t)(G - 1);
-        const uint32_t pos = ((uint32_t)j - h) & (uint32_t)(G - 1);
-        const unsigned before = (1u << pos) - 1u;
-        const uint64_t t = t0 + pos;
-        const bool valid = active && t < A;
-        const uint32_t nv = !active || t0 >= A ? 0u : (A - t0 < (uint64_t)G ? (uint32_t)(A - t0) : (uint32_t)G);
-        uint32_t an = a, bn = b;
-        if (active && t + G < A) {
-            an = __ldcg(S + kn);
-            bn = __ldcg(S + N + mn);
-        }
-        uint32_t kq, mq, r2q;
-        draw(t + 2 * G, kq, mq, r2q);
-        if (active && t + 2 * G < A) {
-            asm volatile("prefetch.L2 [%0];" ::"l"(S + kq));
-            asm volatile("prefetch.L2 [%0];" ::"l"(S + N + mq));
-        }
-        uint32_t na[NS], nb[NS];
-        neighbours<D>(sz, a, na);
-        neighbours<D>(sz, b, nb);
-        uint32_t adj4 = 0;
+        begin();
+        // After a round with many accepted moves, every pair of slots is tried
+        // ahead of the recurrence, slot s against the W / 2 behind it in the
+        // ring; after one with few, only the accepted ones are tried, after it.
+        unsigned behind = 0;       // places of the touched ones
+        if (many) {
+            uint32_t pa[W / 2], pb[W / 2];
+            __syncwarp(FULL);
+            stage[j] = PAIR ? (a | (b << 16)) : a;
+            __syncwarp(FULL);
 #pragma unroll
-        for (int i = 0; i < NS; ++i) adj4 |= (na[i] == b) ? 4u : 0u;
-        const int d4 = v.d4(a, b, na, nb) + (int)adj4;
-        const int de4 = valid ? d4 : 0;
-        // every pair of lanes once, lane l with lane l + d: bit l of ballot d
-        // tells whether their moves touch
-        unsigned cm = 0;
-#pragma unroll
-        for (int d = 1; d <= G / 2; ++d) {
-            uint32_t pa, pb;
-            shfl_pair<IdxT>(a, b, gbase + ((j + d) & (G - 1)), pa, pb);
-            bool c = (pa == a) | (pb == b);
-#pragma unroll
-            for (int i = 0; i < NS; ++i)
-                c |= (na[i] == pa) | (na[i] == pb) | (nb[i] == pa) | (nb[i] == pb);
-            const unsigned B = (__ballot_sync(FULL, c) & gm) >> gbase;
-            cm |= B & (1u << ((j - d) & (G - 1)));
-            cm |= ((B >> j) & 1u) << ((j + d) & (G - 1));
-        }
-        cm = turned(cm, h) & before;
-        // the recurrence
-        unsigned am = 0;          // accepted attempts, by place in the window
-        int x0 = 0;
-        if constexpr (TM == kThrShared) {
-            const uint32_t d_own = valid ? (uint32_t)de4 : DEAD;
-            uint32_t row = rbase + (uint32_t)bin * (4u * TS);
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-                const uint32_t di = __shfl_sync(FULL, d_own, (int)h + i, G);
-                const uint32_t ri = __shfl_sync(FULL, r2p, (int)h + i, G);
-                uint32_t T;
-                asm("ld.shared.u32 %0, [%1];" : "=r"(T) : "r"(row + di));
-                const bool ok = T >= ri;
-                row += ok ? di * (uint32_t)TS : 0u;
-                am |= ok ? 1u << i : 0u;
+            for (int d = 1; d <= W / 2; ++d) {
+                const uint32_t x = stage[(j + d) & WM];
+                pa[d - 1] = PAIR ? (x & 0xFFFFu) : x;
+                pb[d - 1] = PAIR ? (x >> 16) : 0u;
             }
-        } else if constexpr (TM == kThrWindow) {
-            const uint32_t d_own = valid ? (uint32_t)de4 : DEAD;
-            int x = bin;
+            if constexpr (!PAIR) {
+                __syncwarp(FULL);
+                stage[j] = b;
+                __syncwarp(FULL);
 #pragma unroll
-            for (int i = 0; i < G; ++i) {
-                const uint32_t di = __shfl_sync(FULL, d_own, (int)h + i, G);
-                const uint32_t ri = __shfl_sync(FULL, r2p, (int)h + i, G);
-                uint32_t T;
-                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(T)
-                             : "r"(((uint32_t)x & (kThrWindowRows - 1u)) * (4u * TS) + (ring_s + 8u * D + di)));
-                const bool ok = T >= ri;
-                x += ok ? (int)di >> 2 : 0;
-                am |= ok ? 1u << i : 0u;
+                for (int d = 1; d <= W / 2; ++d) pb[d - 1] = stage[(j + d) & WM];
             }
+            recurrence();      // (the comparisons below fill its waits too)
+            unsigned c = 0;
+#pragma unroll
+            for (int d = 1; d <= W / 2; ++d)
+                or_if_touch<D>(c, 1u << (d - 1), na, nb, a, b, pa[d - 1], pb[d - 1]);
+            behind = turn_left<W>(c, place + 1);
         } else {
-            const int e0 = (bin + kThrTPad - kScanReach) & ~3;
-            x0 = bin + kThrTPad - e0;
-            const uint4 *q = reinterpret_cast<const uint4 *>(
-                thr + ((uint32_t)((de4 >> 2) + 2 * D) * pitch + (uint32_t)e0));
-            uint32_t ok[kScanWords / 8];
+            recurrence();
+        }
+        prefetch();
+        // the energy bin after the own attempt
+        __syncwarp(FULL);
+        if (j == 0) {
 #pragma unroll
-            for (int g = 0; g < kScanWords / 8; ++g) {
-                const uint4 u = __ldg(q + 2 * g), u2 = __ldg(q + 2 * g + 1);
-                const uint32_t tv[8] = {u.x, u.y, u.z, u.w, u2.x, u2.y, u2.z, u2.w};
-                ok[g] = 0;
-#pragma unroll
-                for (int o = 0; o < 8; ++o) ok[g] |= tv[o] >= r2p ? 1u << (8 * g + o) : 0u;
+            for (int i = 0; i < W; i += 4)
+                *reinterpret_cast<int4 *>(stage + i) = make_int4(xs[i], xs[i + 1], xs[i + 2], xs[i + 3]);
+        }
+        __syncwarp(FULL);
+        const int x1 = (int)stage[place];
+        // attempts that have to wait (bad) and those whose move changes the
+        // energy (up), by place, over the group
+        const unsigned bit = 1u << place;
+        const int de = (int)code - 2 * D;
+        const bool yes = (am & bit) != 0u && place < near;
+        const int x = x1 - (yes ? de : 0);
+        unsigned bad = 0, up = yes && de != 0 ? bit : 0u;
+        if constexpr (TM == kThrGlobal) bad |= (uint32_t)(x - bin + x0) >= (uint32_t)kScanWords ? bit : 0u;
+        if constexpr (TM == kThrWindow) bad |= x < vlo || x > vhi ? bit : 0u;
+        am &= places();
+        if (many) {
+            bad |= (behind & am & (bit - 1u)) ? bit : 0u;
+            bad |= yes ? behind & ~(bit | (bit - 1u)) : 0u;
+        } else {
+            unsigned todo = am;
+            while (__any_sync(FULL, todo != 0u)) {
+                const uint32_t i = todo ? (uint32_t)__ffs(todo) - 1u : 0u;
+                const uint32_t slot = (i + h) & WM;
+                uint32_t pa, pb;
+                shfl_pair<IdxT>(a, b, gbase + (int)slot, pa, pb);
+                or_if_touch<D>(bad, todo != 0u && place > i ? bit : 0u, na, nb, a, b, pa, pb);
+                todo &= todo - 1u;
             }
-            const uint32_t word = ((uint32_t)(de4 >> 2) << 24) | (valid ? ok[0] | ok[1] | ok[2] : 0u);
-            int x = x0;
+        }
+        if constexpr (W <= 16) {
+            unsigned y = bad | (up << 16);
 #pragma unroll
-            for (int i = 0; i < G; ++i) {
-                const uint32_t wi = __shfl_sync(FULL, word, (int)h + i, G);
-                const bool yes = (__funnelshift_r(wi, wi, (uint32_t)x) & 1u) != 0u;
-                x += yes ? (int)wi >> 24 : 0;
-                am |= yes ? 1u << i : 0u;
+            for (int o = 1; o < W; o <<= 1) y |= __shfl_xor_sync(FULL, y, o);
+            bad = y & 0xFFFFu;
+            up = y >> 16;
+        } else {
+#pragma unroll
+            for (int o = 1; o < W; o <<= 1) {
+                bad |= __shfl_xor_sync(FULL, bad, o);
+                up |= __shfl_xor_sync(FULL, up, o);
             }
         }
-        // the energy after this lane's attempt is bin + incl
-        const int de = de4 >> 2;
-        const bool yes = valid && ((am >> pos) & 1u);
-        int incl = yes ? de : 0;
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-            const int y = __shfl_sync(FULL, incl, (j - o) & (G - 1), G);
-            incl += pos >= (uint32_t)o ? y : 0;
-        }
-        bool bad = (cm & am) != 0u;
-        if constexpr (TM == kThrGlobal)
-            bad = bad || (uint32_t)(x0 + incl - (yes ? de : 0)) >= (uint32_t)kScanWords;
-        if constexpr (TM == kThrWindow) {
-            const int e = bin + incl - (yes ? de : 0);
-            bad = bad || e < vlo || e > vhi;
-        }
-        const unsigned bb = turned((__ballot_sync(FULL, valid && bad) & gm) >> gbase, h);
-        const uint32_t nd = bb ? (uint32_t)__ffs(bb) - 1u : nv;    // attempts decided
-        const bool decided = pos < nd;
-        const bool commit = yes && decided;
-        const unsigned chg = turned((__ballot_sync(FULL, commit && de != 0) & gm) >> gbase, h);
+        // attempts decided (a bad one past the end is none)
+        const uint32_t nv = near < W ? near : (uint32_t)W;
+        const uint32_t nd = bad ? min((uint32_t)__ffs(bad) - 1u, nv) : nv;
+        const unsigned done = W == 32 && nd >= 32u ? 0xffffffffu : (1u << nd) - 1u;
+        const unsigned chg = up & done;
+        many = __any_sync(FULL, __popc(am) > kScanFew);
+        quiet = false;
+        if (!many) quiet = !__any_sync(FULL, am != 0u);
+        const bool commit = yes && place < nd;
+        // the list slots a commit rewrites
+        const uint32_t moved = commit && PAIR ? (k | (m << 16)) : 0xFFFFFFFFu;   // (indices below 65535)
         if (commit) {
             v.commit(a, b, na, nb);
             S[k] = (IdxT)b;
             S[N + m] = (IdxT)a;
             ++acc;
             // a move ends the run at the energy before it
-            const unsigned prev = chg & before;
-            const uint32_t cnt = prev ? pos - 31u + (uint32_t)__clz(prev) : carry + pos;
-            if (de != 0 && cnt != 0u) atomicAdd(hist + (bin + incl - de), (unsigned long long)cnt);
+            const unsigned prev = chg & (bit - 1u);
+            const uint32_t cnt = prev ? place - 31u + (uint32_t)__clz(prev) : carry + place;
+            if (de != 0 && cnt != 0u) atomicAdd(hist + (x1 - de), (unsigned long long)cnt);
         }
         carry = chg ? nd - 31u + (uint32_t)__clz(chg) : carry + nd;
         if (tun) {      // (the same in the whole block)
-            unsigned tl = turned((__ballot_sync(FULL, commit && bin + incl <= tlo) & gm) >> gbase, h);
-            unsigned th = turned((__ballot_sync(FULL, commit && bin + incl >= thi) & gm) >> gbase, h);
+            unsigned tl = commit && x1 <= tlo ? bit : 0u;
+            unsigned th = commit && x1 >= thi ? bit : 0u;
+#pragma unroll
+            for (int o = 1; o < W; o <<= 1) {
+                tl |= __shfl_xor_sync(FULL, tl, o);
+                th |= __shfl_xor_sync(FULL, th, o);
+            }
             while (tl | th) {      // events in attempt order, runs of one end at once
                 if (th == 0u || (tl != 0u && __ffs(tl) < __ffs(th))) {
                     tcnt += tst == 2u ? 1u : 0u;
@@ -358,43 +548,48 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
             }
             __syncwarp(FULL);
         }
-        // (with nd = 0 no attempt is left and every lane's incl is 0)
-        bin += __shfl_sync(FULL, incl, (int)(h + nd) - 1, G);
-        // what this lane goes on with: its next attempt, or the same one again
+        // the energy the window goes on from: after its last decided attempt
+        bin = nd ? (int)stage[nd - 1u] : bin;
         const uint32_t a_i = a, b_i = b, k_i = k, m_i = m;
-        k = decided ? kn : k;
-        m = decided ? mn : m;
-        a = decided ? an : a;
-        b = decided ? bn : b;
-        r2p = decided ? r2n : r2p;
-        kn = decided ? kq : kn;
-        mn = decided ? mq : mn;
-        r2n = decided ? r2q : r2n;
+        advance(place < nd);
         // its list entries, read before this round's commits, where a commit
         // moved one of its slots (at most one commit of a round per slot)
-        bool hit = false;
-        const uint32_t s_i = commit ? k_i : 0xFFFFFFFFu, t_i = commit ? m_i : 0xFFFFFFFFu;
-        if constexpr (sizeof(IdxT) == 2) {
-            const uint32_t slots = (s_i & 0xFFFFu) | (t_i << 16);   // slot indices are below 65535
+        if constexpr (PAIR) {
+            __syncwarp(FULL);
+            stage[j] = moved;
+            __syncwarp(FULL);
+            uint32_t ms[W];
+#pragma unroll
+            for (int i = 0; i < W; i += 4) *reinterpret_cast<uint4 *>(ms + i) = *reinterpret_cast<const uint4 *>(stage + i);
             const uint32_t own = k | (m << 16);
-            uint32_t low = 0xFFFFFFFFu;      // the least of each half over the lanes
+            uint32_t low = 0xFFFFFFFFu;     // the least of each half
 #pragma unroll
-            for (int i = 0; i < G; ++i) low = __vminu2(low, __shfl_sync(FULL, slots, i, G) ^ own);
-            hit = (low & 0xFFFFu) == 0u || low < 0x10000u;
-        } else {
+            for (int i = 0; i < W; i += 2) low = __vimin3_u16x2(low, ms[i] ^ own, ms[i + 1] ^ own);
+            if (__any_sync(FULL, (low & 0xFFFFu) == 0u || low < 0x10000u)) {
+                int of_k = -1, of_m = -1;
 #pragma unroll
-            for (int i = 0; i < G; ++i) {
-                const uint32_t ki = __shfl_sync(FULL, s_i, i, G), mi = __shfl_sync(FULL, t_i, i, G);
-                hit = hit || ki == k || mi == m;
+                for (int i = 0; i < W; ++i) {
+                    const uint32_t x = ms[i] ^ (k | (m << 16));
+                    of_k = (x & 0xFFFFu) == 0u ? i : of_k;
+                    of_m = x < 0x10000u ? i : of_m;
+                }
+                const uint32_t to_k = __shfl_sync(FULL, b_i, of_k & (W - 1), W);
+                const uint32_t to_m = __shfl_sync(FULL, a_i, of_m & (W - 1), W);
+                a = of_k >= 0 ? to_k : a;
+                b = of_m >= 0 ? to_m : b;
             }
-        }
-        if (__any_sync(FULL, hit)) {
+        } else {
+            if (__any_sync(FULL, commit)) {
 #pragma unroll
-            for (int i = 0; i < G; ++i) {
-                const uint32_t ki = __shfl_sync(FULL, s_i, i, G), mi = __shfl_sync(FULL, t_i, i, G);
-                const uint32_t ai = __shfl_sync(FULL, a_i, i, G), bi = __shfl_sync(FULL, b_i, i, G);
-                a = ki == k ? bi : a;
-                b = mi == m ? ai : b;
+                for (int i = 0; i < W; ++i) {
+                    const bool ci = __shfl_sync(FULL, (int)commit, i, W) != 0;
+                    const uint32_t ki = __shfl_sync(FULL, k_i, i, W);
+                    const uint32_t mi = __shfl_sync(FULL, m_i, i, W);
+                    const uint32_t ai = __shfl_sync(FULL, a_i, i, W);
+                    const uint32_t bi = __shfl_sync(FULL, b_i, i, W);
+                    a = ci && ki == k ? bi : a;
+                    b = ci && mi == m ? ai : b;
+                }
             }
         }
         t0 += nd;
@@ -418,7 +613,7 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
         }
     }
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    for (int o = W / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
     if (active && j == 0) {
         if (carry) atomicAdd(hist + bin, (unsigned long long)carry);
         p.E[w] = bin + p.e_lo;
@@ -433,11 +628,11 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
 // How the rounds read a walker's occupation.
 enum ScanView { kViewBitsShared, kViewBitsGlobal, kViewField };
 
-template <int D, typename IdxT, int G, int TM, int VIEW>
+template <int D, typename IdxT, int W, int TM, int VIEW>
 __device__ __forceinline__ void scan_item(const SysParams &p, const BlockWork &wk, uint32_t *smem,
-                                          uint64_t sweeps, uint32_t iter)
+                                          uint32_t *stage, uint64_t sweeps, uint32_t iter)
 {
-    const int lw = threadIdx.x / G;
+    const int lw = threadIdx.x / W;
     const bool active = lw < wk.count;
     const int w = wk.walker0 + (active ? lw : 0);
     const uint32_t *thr = TM == kThrShared ? smem : (TM == kThrWindow ? p.thr : p.thrT);
@@ -446,10 +641,10 @@ __device__ __forceinline__ void scan_item(const SysParams &p, const BlockWork &w
     uint32_t *state = smem + (TM == kThrShared ? thr_words_aligned(p) : 0);
     uint32_t ring_s = 0u, mbar_s = 0u;
     if constexpr (TM == kThrWindow) {
-        const uint32_t wpb = blockDim.x / G;
-        const uint32_t used = VIEW == kViewField ? wpb * (uint32_t)field_bytes(p)
-                              : VIEW == kViewBitsShared ? wpb * (uint32_t)p.words * 4u : 0u;
-        window_addrs(p, (uint32_t)__cvta_generic_to_shared(state) + used, (int)wpb, active ? lw : 0,
+        const int wpb = (int)blockDim.x / W;
+        const uint32_t used = VIEW == kViewField ? (uint32_t)wpb * (uint32_t)field_bytes(p)
+                              : VIEW == kViewBitsShared ? (uint32_t)wpb * (uint32_t)p.words * 4u : 0u;
+        window_addrs(p, (uint32_t)__cvta_generic_to_shared(state) + used, wpb, active ? lw : 0,
                      ring_s, mbar_s);
     }
     if constexpr (VIEW == kViewField) {
@@ -457,37 +652,38 @@ __device__ __forceinline__ void scan_item(const SysParams &p, const BlockWork &w
         field_build<D, IdxT>(p, wk, state);   // ends with a block barrier, which also covers the table
         const ScanField<D> v{(uint32_t)__cvta_generic_to_shared(state) +
                              (uint32_t)((size_t)(active ? lw : 0) * field_bytes(p))};
-        chain_scan<D, IdxT, G, TM>(p, w, active, v, thr, hist, A, iter, ring_s, mbar_s);
+        chain_scan<D, IdxT, W, TM>(p, w, active, v, thr, hist, A, iter, ring_s, mbar_s, stage);
         field_finish<IdxT>(p, wk, state);
     } else {
         constexpr bool SB = VIEW == kViewBitsShared;
         const BlockSetup bs = block_setup(p, wk, smem, SB ? 1 : 0, TM == kThrShared ? 1 : 0);
         uint32_t *bits0 = SB ? state : p.bits + (size_t)wk.walker0 * (size_t)p.words;
         const ScanBits<D, SB> v{bits0 + (size_t)(active ? lw : 0) * p.words};
-        chain_scan<D, IdxT, G, TM>(p, w, active, v, thr, hist, A, iter, ring_s, mbar_s);
+        chain_scan<D, IdxT, W, TM>(p, w, active, v, thr, hist, A, iter, ring_s, mbar_s, stage);
         block_finish(bs, SB ? 1 : 0);
     }
 }
 
 // Block b takes work item b; with a counter (persistent launches), then the
 // items that it pulls from it.
-template <int G, int TM, int VIEW>
+template <int W, int TM, int VIEW>
 __global__ void __launch_bounds__(kGroupMaxThreads, 1)
 walker_update_scan(const SysParams *__restrict__ sys, const BlockWork *__restrict__ work,
                    uint64_t sweeps, uint32_t iter, int n_items, int *next_item)
 {
     extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ __align__(16) uint32_t stage[kGroupMaxThreads];
     __shared__ int s_item;
     int item = blockIdx.x;
     for (;;) {
         const BlockWork wk = work[item];
         const SysParams &p = sys[wk.sys];
         if (p.d == 2) {
-            if (p.idx16) scan_item<2, uint16_t, G, TM, VIEW>(p, wk, smem, sweeps, iter);
-            else scan_item<2, uint32_t, G, TM, VIEW>(p, wk, smem, sweeps, iter);
+            if (p.idx16) scan_item<2, uint16_t, W, TM, VIEW>(p, wk, smem, stage, sweeps, iter);
+            else scan_item<2, uint32_t, W, TM, VIEW>(p, wk, smem, stage, sweeps, iter);
         } else {
-            if (p.idx16) scan_item<3, uint16_t, G, TM, VIEW>(p, wk, smem, sweeps, iter);
-            else scan_item<3, uint32_t, G, TM, VIEW>(p, wk, smem, sweeps, iter);
+            if (p.idx16) scan_item<3, uint16_t, W, TM, VIEW>(p, wk, smem, stage, sweeps, iter);
+            else scan_item<3, uint32_t, W, TM, VIEW>(p, wk, smem, stage, sweeps, iter);
         }
         if (!next_item) break;
         item = next_work_item(next_item, &s_item);
