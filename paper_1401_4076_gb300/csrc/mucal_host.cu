@@ -41,6 +41,8 @@ struct System {
     uint64_t last_attempts = 0;
     std::vector<double> lnW_run;    // the weights of the last iteration's thresholds
     unsigned long long *drop_acc = nullptr;  // device [3][n_bins] droplet accumulators
+    mucal::DropletPlan drop_plan{};          // of its droplet measurement, once made
+    bool drop_planned = false;
     int32_t *drop_last = nullptr;            // device [n_walkers] V_D of the last measurement
 };
 
@@ -1430,11 +1432,11 @@ int mucal_measure_droplets(void *ctx)
     Context *c = as_ctx(ctx);
     if (!c) return MUCAL_ERR_INVALID_ARG;
     CUDA_TRY(c, cudaSetDevice(c->device));
-    std::vector<mucal::DropletPlan> plans(c->sys.size());
     size_t scratch = 0;
-    for (size_t i = 0; i < c->sys.size(); ++i) {
-        CUDA_TRY(c, mucal::droplet_plan(c->sys[i].p, &plans[i]));
-        scratch = std::max(scratch, plans[i].scratch_words);
+    for (auto &s : c->sys) {
+        if (!s.drop_planned) CUDA_TRY(c, mucal::droplet_plan(s.p, &s.drop_plan));
+        s.drop_planned = true;
+        scratch = std::max(scratch, s.drop_plan.scratch_words);
     }
     if (scratch > c->drop_scratch_words) {
         // the previous scratch may still be read by an earlier measurement
@@ -1448,7 +1450,7 @@ int mucal_measure_droplets(void *ctx)
     for (size_t i = 0; i < c->sys.size(); ++i) {
         const System &s = c->sys[i];
         const mucal::DropletOut o{s.drop_acc, s.drop_last, c->d_drop_err};
-        CUDA_TRY(c, mucal::launch_droplets(s.p, o, plans[i], c->drop_scratch, c->stream));
+        CUDA_TRY(c, mucal::launch_droplets(s.p, o, s.drop_plan, c->drop_scratch, c->stream));
     }
     c->measured = true;
     return MUCAL_OK;

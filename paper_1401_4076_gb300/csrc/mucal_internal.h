@@ -152,8 +152,10 @@ struct DropletOut {
     int *err;                  // set non-zero on a labelling or energy-range failure
 };
 struct DropletPlan {
-    bool shared;               // parent array in shared memory (else global scratch)
+    bool rank;                 // tables by particle rank (droplet_rank_kernel)
+    bool shared;               // else: parent array in shared memory (else global scratch)
     int grid;                  // blocks; each strides over the walkers
+    int threads;               // threads per block (rank)
     size_t smem;               // dynamic shared memory per block
     size_t scratch_words;      // uint32 words of global scratch the launch needs
 };

@@ -86,6 +86,25 @@ def test_largest_droplet_bit_exact(desc, kind, rounds, sweeps):
         assert max(g.max() for g in got) >= desc[2] // 2   # droplets really formed
 
 
+@pytest.mark.parametrize("desc,kind,rounds,sweeps", [
+    ((2, 31, 300, 9, 0, 0, 2), "condense", 2, 20),        # rows that start inside words, ragged last word
+    ((2, 33, 1000, 5, 0, 0, 4), "random", 1, 2),          # long runs along the rows, odd N
+    ((3, 16, 1500, 7, 0, 0, 6), "condense", 1, 5),        # 128 words: the wider blocks
+    ((2, 128, 1638, 3, 0, 0, 7), "condense", 1, 5),       # 512 words: the widest
+    ((2, 257, 1001, 2, 0, 0, 8), "condense", 1, 5),       # uint32 sites and counters, odd N
+    ((2, 230, 38000, 2, 0, 0, 9), "random", 1, 1),        # tables by rank too large: parents per site
+    ((3, 40, 40000, 2, 0, 0, 10), "random", 1, 1),        # ... and those too: global parents
+])
+def test_droplet_tables_bit_exact(desc, kind, rounds, sweeps):
+    """The sizes at which the labelling changes its tables, and rows that do
+    not line up with the bitset's words."""
+    got, want, dev, acc = _run_both(desc, kind, rounds, sweeps)
+    for g, w in zip(got, want):
+        np.testing.assert_array_equal(g, w)
+    for k in range(3):
+        np.testing.assert_array_equal(dev[k], acc[k])
+
+
 @pytest.mark.parametrize("wl,sweeps", [(workloads.MEDIUM_2D, 20), (workloads.LARGE_3D, 2)])
 def test_droplet_full_size(wl, sweeps):
     """The 64x64 (N = 410, 4096 walkers) and 32^3 (N = 3277, 8192 walkers)
