@@ -38,6 +38,7 @@ struct System {
     bool target_default = true;
     uint32_t *thr_pinned = nullptr; // staging buffer of the threshold upload
     size_t thr_count = 0;
+    size_t hist_cap = 0;            // histogram rows allocated
     uint64_t last_attempts = 0;
     std::vector<double> lnW_run;    // the weights of the last iteration's thresholds
     unsigned long long *drop_acc = nullptr;  // device [3][n_bins] droplet accumulators
@@ -376,9 +377,14 @@ size_t smem_for(const LaunchShape &sh, const SysParams &p)
     return bytes;
 }
 
+void drop_graph(Context *c);
+
 // Split every system's walkers into blocks of the launch shape; order the
 // blocks by decreasing cost (attempts per walker grow with N) so the longest
-// blocks start first when systems of uneven size share one launch.
+// blocks start first when systems of uneven size share one launch.  The
+// histogram rows are allocated here, as many as the shape needs (one per
+// block: 23 MB instead of one per walker, 644 MB, on 3D L = 32 with 8192
+// walkers), and grow when a shape needs more.
 int build_work(Context *c, const LaunchShape &sh)
 {
     std::vector<BlockWork> work;
@@ -411,14 +417,20 @@ int build_work(Context *c, const LaunchShape &sh)
     if (e == cudaSuccess)
         e = cudaMemcpy(d_work, work.data(), work.size() * sizeof(BlockWork), cudaMemcpyHostToDevice);
     std::vector<SysParams> hp(c->sys.size());
+    std::vector<void *> grown(c->sys.size(), nullptr);
     for (size_t i = 0; i < c->sys.size(); ++i) {
         hp[i] = c->sys[i].p;
         hp[i].hist_rows = rows_of[i];
+        if (e == cudaSuccess && (size_t)rows_of[i] > c->sys[i].hist_cap) {
+            e = cudaMalloc(&grown[i], (size_t)rows_of[i] * (size_t)hp[i].n_bins * 8);
+            hp[i].hist = static_cast<unsigned long long *>(grown[i]);
+        }
     }
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_sys, hp.data(), hp.size() * sizeof(SysParams), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(d_work);
+        for (void *q : grown) cudaFree(q);
         // restore the device table of the current shape
         std::vector<SysParams> cur(c->sys.size());
         for (size_t i = 0; i < c->sys.size(); ++i) cur[i] = c->sys[i].p;
@@ -429,7 +441,14 @@ int build_work(Context *c, const LaunchShape &sh)
     cudaFree(c->d_work);
     c->d_work = d_work;
     c->n_blocks = (int)work.size();
-    for (size_t i = 0; i < c->sys.size(); ++i) c->sys[i].p.hist_rows = rows_of[i];
+    for (size_t i = 0; i < c->sys.size(); ++i) {
+        c->sys[i].p.hist_rows = rows_of[i];
+        if (!grown[i]) continue;
+        drop_graph(c);               // a captured iteration holds the old rows
+        cudaFree(c->sys[i].p.hist);
+        c->sys[i].p.hist = hp[i].hist;
+        c->sys[i].hist_cap = (size_t)rows_of[i];
+    }
     return MUCAL_OK;
 }
 
@@ -520,7 +539,7 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
 // L = 14, N = 17, r = 19: 0.51 / 0.65 / 1.40 / -.
 int default_lanes(long long r, double N)
 {
-    if (N < 32 || (N < 200 && r > 40)) return 4;
+    if (N < 32 || (N < 200 && r > 48)) return 4;
     if (N >= 2500 && r <= 7) return 32;
     if ((N >= 1000 && r <= 24) || (N >= 300 && r <= 4)) return 16;
     return 8;
@@ -861,7 +880,6 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
         ALLOC(bits, nw * p.words * sizeof(uint32_t));
         ALLOC(S, nw * (size_t)p.V * ib);
         ALLOC(E, nw * sizeof(int32_t));
-        ALLOC(hist, nw * (size_t)p.n_bins * sizeof(unsigned long long));
         ALLOC(thr, (size_t)p.n_bins * p.tstride * sizeof(uint32_t));
         ALLOC(accepts, nw * sizeof(unsigned long long));
         ALLOC(H, (size_t)p.n_bins * sizeof(unsigned long long));
@@ -894,7 +912,6 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
             cudaMemsetAsync(s.drop_last, 0, nw * sizeof(int32_t), c->stream) != cudaSuccess)
             return bail(fail(nullptr, MUCAL_ERR_CUDA, "memset failed"));
         if (cudaMemsetAsync(p.bits, 0, nw * p.words * sizeof(uint32_t), c->stream) != cudaSuccess ||
-            cudaMemsetAsync(p.hist, 0, nw * (size_t)p.n_bins * 8, c->stream) != cudaSuccess ||
             cudaMemsetAsync(p.H, 0, (size_t)p.n_bins * 8, c->stream) != cudaSuccess ||
             cudaMemsetAsync(p.accepts, 0, nw * 8, c->stream) != cudaSuccess ||
             cudaMemsetAsync(p.tun_state, 0, nw, c->stream) != cudaSuccess ||
@@ -919,8 +936,7 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
     for (int i = 0; i < n_sys; ++i) hp[i] = c->sys[i].p;
     if (cudaMemcpy(c->d_sys, hp.data(), n_sys * sizeof(SysParams), cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(fail(nullptr, MUCAL_ERR_CUDA, "copy of system table failed"));
-    if (mucal::launch_fill_identity(hp.data(), c->d_sys, n_sys, c->stream) != cudaSuccess ||
-        mucal::launch_init_walkers(hp.data(), c->d_sys, n_sys, c->stream) != cudaSuccess)
+    if (mucal::launch_init_walkers(hp.data(), n_sys, c->stream) != cudaSuccess)
         return bail(fail(nullptr, MUCAL_ERR_CUDA, "initial placement launch failed"));
     for (int i = 0; i < n_sys; ++i) {
         rc = upload_thresholds(c, c->sys[i]);

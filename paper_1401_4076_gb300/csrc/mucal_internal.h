@@ -91,10 +91,8 @@ struct LaunchShape {
 };
 
 // Kernel launchers (walker_kernels.cu).  All are asynchronous on `stream`.
-cudaError_t launch_fill_identity(const SysParams *host_sys, const SysParams *dev_sys, int n_sys,
-                                 cudaStream_t stream);
-cudaError_t launch_init_walkers(const SysParams *host_sys, const SysParams *dev_sys, int n_sys,
-                                cudaStream_t stream);
+// Place every walker's particles: site lists, bitsets (zero before) and energies.
+cudaError_t launch_init_walkers(const SysParams *host_sys, int n_sys, cudaStream_t stream);
 // The walker-update kernel of a launch shape; tunnel selects the flavour with
 // the tunnelling bookkeeping (Sec. 4).  Its arguments are (const SysParams *,
 // const BlockWork *, uint64_t sweeps, uint32_t iteration, int n_items,

@@ -86,11 +86,6 @@ __device__ __forceinline__ void neighbours(const Lattice &p, uint32_t s, uint32_
     }
 }
 
-__device__ __forceinline__ uint32_t occupied(const uint32_t *bits, uint32_t s)
-{
-    return (bits[s >> 5] >> (s & 31u)) & 1u;
-}
-
 template <typename IdxT>
 __device__ __forceinline__ IdxT *walker_S(const SysParams &p, int w)
 {

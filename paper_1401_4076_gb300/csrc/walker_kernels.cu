@@ -19,62 +19,174 @@
 namespace mucal {
 namespace {
 // ---------------------------------------------------------------------------
-// Initial placement.
+// Initial placement: a partial Fisher-Yates shuffle of the site list from the
+// init stream (step j swaps S[j] with S[j + floor(r (V - j) / 2^32)], r = word
+// j % 4 of the block with counter (j/4 lo, j/4 hi, 0, 1)), then the bitset and
+// a full energy count over the particles, looking in the +1 direction of
+// every axis so each bond counts once.
+//
+// One block places one walker, and 32 steps of the shuffle are taken at once
+// by its first warp: step m of such a batch has to wait for an earlier step l
+// of it only if l's target is m's position or m's target.  The block looks for
+// such steps in all batches first (0.72 -> 0.54 ms), and a batch that holds one
+// (3D L = 32: one in twenty) is taken in parts.  Where the list fits into
+// shared memory the shuffle runs there and the list is written once, in order;
+// a list in global memory costs a random access per swap.  Bound by the first
+// warp's chain of batches, three blocks to an SM by the lists' 64 KB; the
+// write alone would take 0.08 ms.  8192 walkers of 3D L = 32, N = 3277 (537 MB
+// of lists): 5.48 ms with one thread per walker on lists in global memory ->
+// 0.54 ms.
 // ---------------------------------------------------------------------------
-template <typename IdxT>
-__global__ void fill_identity(SysParams p)
-{
-    const size_t total = (size_t)p.n_walkers * (size_t)p.V;
-    IdxT *S = reinterpret_cast<IdxT *>(p.S);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x)
-        S[i] = (IdxT)(i % (size_t)p.V);
-}
+constexpr int kInitThreads = 128;
+constexpr int kInitChunk = 1024;        // targets drawn at a time, by the whole block
 
-// Partial Fisher-Yates from the init stream (counter (j/4 lo, j/4 hi, 0, 1),
-// word j%4), then the bitset and a full energy count over the particles,
-// looking in the +1 direction of every axis so each bond counts once.
-template <int D, typename IdxT>
-__device__ void init_one(const SysParams &p, int w)
+template <int D, typename IdxT, bool SMEM>
+__global__ void __launch_bounds__(kInitThreads)
+init_place_kernel(SysParams p, int bits_in_smem)
 {
-    IdxT *S = walker_S<IdxT>(p, w);
-    const uint64_t seed = p.seed_base + (uint64_t)w;
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    const uint32_t V = (uint32_t)p.V;
-    uint4 r = make_uint4(0, 0, 0, 0);
-    for (uint32_t j = 0; j < (uint32_t)p.N; ++j) {
-        if ((j & 3u) == 0) r = philox10(make_uint4(j >> 2, 0u, 0u, 1u), k0, k1);
-        const uint32_t word = (j & 3u) == 0 ? r.x : (j & 3u) == 1 ? r.y : (j & 3u) == 2 ? r.z : r.w;
-        const uint32_t idx = j + __umulhi(word, V - j);
-        const IdxT tmp = S[j];
-        S[j] = S[idx];
-        S[idx] = tmp;
-    }
-    uint32_t *bits = p.bits + (size_t)w * (size_t)p.words;
-    for (uint32_t j = 0; j < (uint32_t)p.N; ++j) {
-        const uint32_t s = S[j];
-        bits[s >> 5] |= 1u << (s & 31u);
-    }
-    int pairs = 0;
-    for (uint32_t j = 0; j < (uint32_t)p.N; ++j) {
-        uint32_t nb[2 * D];
-        neighbours<D>(p, (uint32_t)S[j], nb);
+    extern __shared__ __align__(16) uint32_t dyn[];
+    __shared__ uint32_t target[kInitChunk];
+    __shared__ unsigned waits[kInitChunk / 32];
+    __shared__ int red[kInitThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t V = (uint32_t)p.V, N = (uint32_t)p.N;
+    for (int w = blockIdx.x; w < p.n_walkers; w += gridDim.x) {
+        IdxT *out = walker_S<IdxT>(p, w);
+        uint32_t *gbits = p.bits + (size_t)w * (size_t)p.words;
+        uint32_t *bits = bits_in_smem ? dyn : gbits;      // (global bitsets start at zero)
+        volatile IdxT *S = out;
+        if constexpr (SMEM) S = reinterpret_cast<IdxT *>(dyn + ((p.words + 3) & ~3));
+        const uint64_t seed = p.seed_base + (uint64_t)w;
+        const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+        if constexpr (SMEM) {
+            // (the shared list is rounded up to 16 bytes)
+            constexpr uint32_t PER = 16u / sizeof(IdxT);
+            uint4 *s4 = reinterpret_cast<uint4 *>(dyn + ((p.words + 3) & ~3));
+            for (uint32_t i = tid; i * PER < V; i += kInitThreads) {
+                const uint32_t v = i * PER;
+                s4[i] = sizeof(IdxT) == 2 ? make_uint4(v | ((v + 1) << 16), (v + 2) | ((v + 3) << 16),
+                                                       (v + 4) | ((v + 5) << 16), (v + 6) | ((v + 7) << 16))
+                                          : make_uint4(v, v + 1, v + 2, v + 3);
+            }
+        } else {
+            for (uint32_t i = tid; i < V; i += kInitThreads) S[i] = (IdxT)i;
+        }
+        if (bits_in_smem)
+            for (int i = tid; i < p.words; i += kInitThreads) dyn[i] = 0u;
+        for (uint32_t c = 0; c < N; c += kInitChunk) {
+            const uint32_t end = min(c + (uint32_t)kInitChunk, N);
+            for (uint32_t j = c + 4u * tid; j < end; j += 4u * kInitThreads) {
+                const uint4 r = philox10(make_uint4(j >> 2, 0u, 0u, 1u), k0, k1);
+                const uint32_t word[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-        for (int k = 0; k < D; ++k) pairs += (int)occupied(bits, nb[2 * k + 1]);
+                for (uint32_t q = 0; q < 4; ++q)
+                    if (j + q < end) target[j + q - c] = j + q + __umulhi(word[q], V - (j + q));
+            }
+            __syncthreads();
+            // steps of [j, j + 32) up to end that have to wait for an earlier
+            // one: their position or target is an earlier lane's target
+            auto waiting = [&](uint32_t j, uint32_t stop, uint32_t &t) -> unsigned {
+                const uint32_t me = j + (uint32_t)lane;
+                const bool in = me < stop;
+                t = in ? target[me - c] : 0xFFFFFFFFu - (uint32_t)lane;
+                const unsigned same = __match_any_sync(0xFFFFFFFFu, t) & ((1u << lane) - 1u);
+                const unsigned hits = __reduce_or_sync(0xFFFFFFFFu, in && t > me && t - j < 32u ? 1u << (t - j) : 0u);
+                return hits | __ballot_sync(0xFFFFFFFFu, in && same != 0u);
+            };
+            // the whole block looks every batch over first, so that the chain
+            // of swaps below has only its loads and stores
+            for (uint32_t j = c + 32u * (uint32_t)(tid >> 5); j < end; j += kInitThreads) {
+                uint32_t t;
+                const unsigned wait = waiting(j, end, t);
+                if (lane == 0) waits[(j - c) >> 5] = wait;
+            }
+            __syncthreads();
+            if (tid < 32) {
+                for (uint32_t j0 = c; j0 < end; j0 += 32u) {
+                    unsigned wait = waits[(j0 - c) >> 5];
+                    const uint32_t stop = min(j0 + 32u, end);
+                    uint32_t t = target[min(j0 + (uint32_t)lane, end - 1u) - c];
+                    for (uint32_t j = j0;;) {
+                        const uint32_t n = min(wait ? (uint32_t)__ffs(wait) - 1u : 32u, stop - j);
+                        if ((uint32_t)lane < n) {
+                            const uint32_t me = j + (uint32_t)lane;
+                            const IdxT x = S[me], y = S[t];
+                            S[me] = y;
+                            S[t] = x;
+                        }
+                        __syncwarp();
+                        j += n;
+                        if (j >= stop) break;
+                        wait = waiting(j, stop, t);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        for (uint32_t i = tid; i < N; i += kInitThreads) {
+            const uint32_t s = (uint32_t)S[i];
+            atomicOr(bits + (s >> 5), 1u << (s & 31u));
+        }
+        if constexpr (SMEM) {
+            // (16-byte stores where the walker's list starts on 16 bytes)
+            const IdxT *src = reinterpret_cast<const IdxT *>(dyn + ((p.words + 3) & ~3));
+            const size_t bytes = (size_t)V * sizeof(IdxT);
+            if (((uintptr_t)out & 15u) == 0u) {
+                const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
+                uint4 *o4 = reinterpret_cast<uint4 *>(out);
+                for (size_t i = tid; i < bytes / 16; i += kInitThreads) o4[i] = s4[i];
+                for (size_t i = bytes / 16 * 16 / sizeof(IdxT) + tid; i < V; i += kInitThreads) out[i] = src[i];
+            } else {
+                for (uint32_t i = tid; i < V; i += kInitThreads) out[i] = src[i];
+            }
+        }
+        __syncthreads();
+        int pairs = 0;
+        for (uint32_t i = tid; i < N; i += kInitThreads) {
+            uint32_t nb[2 * D];
+            neighbours<D>(p, (uint32_t)S[i], nb);
+#pragma unroll
+            for (int k = 0; k < D; ++k) {
+                const uint32_t t = nb[2 * k + 1];
+                const uint32_t x = bits_in_smem ? bits[t >> 5] : __ldcg(bits + (t >> 5));
+                pairs += (int)((x >> (t & 31u)) & 1u);
+            }
+        }
+        if (bits_in_smem)
+            for (int i = tid; i < p.words; i += kInitThreads) gbits[i] = dyn[i];
+        pairs = __reduce_add_sync(0xFFFFFFFFu, pairs);
+        if (lane == 0) red[tid >> 5] = pairs;
+        __syncthreads();
+        if (tid == 0) {
+            int e = 0;
+            for (int i = 0; i < kInitThreads / 32; ++i) e -= red[i];
+            p.E[w] = e;
+        }
+        __syncthreads();     // the list, the bitset and red are reused by the next walker
     }
-    p.E[w] = -pairs;
 }
 
-__global__ void init_walkers_kernel(const SysParams *__restrict__ sys, int s)
+template <int D, typename IdxT>
+cudaError_t init_place(const SysParams &p, int optin, int sms, cudaStream_t stream)
 {
-    const SysParams &p = sys[s];
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= p.n_walkers) return;
-    if (p.d == 2) {
-        if (p.idx16) init_one<2, uint16_t>(p, w); else init_one<2, uint32_t>(p, w);
-    } else {
-        if (p.idx16) init_one<3, uint16_t>(p, w); else init_one<3, uint32_t>(p, w);
-    }
+    const size_t bits = (size_t)((p.words + 3) & ~3) * 4, list = ((size_t)p.V * sizeof(IdxT) + 15) & ~(size_t)15;
+    const size_t room = (size_t)optin - 6 * 1024;       // beside the static arrays
+    const bool in_smem = bits + list <= room;
+    const int bits_in_smem = bits <= room ? 1 : 0;
+    const size_t smem = in_smem ? bits + list : (bits_in_smem ? bits : 0);
+    const void *fn = in_smem ? (const void *)init_place_kernel<D, IdxT, true>
+                             : (const void *)init_place_kernel<D, IdxT, false>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+    int per_sm = 0;
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kInitThreads, smem);
+    if (e != cudaSuccess) return e;
+    const long long blocks = (long long)sms * (per_sm > 0 ? per_sm : 1);
+    const int grid = (int)(p.n_walkers < blocks ? p.n_walkers : blocks);
+    SysParams q = p;
+    int flag = bits_in_smem;
+    void *args[] = {(void *)&q, (void *)&flag};
+    return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kInitThreads), args, smem, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -190,37 +302,20 @@ cudaError_t launch_exchange(const SysParams *dev_sys, int n_sys, int n_walkers, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_fill_identity(const SysParams *host_sys, const SysParams *dev_sys, int n_sys,
-                                 cudaStream_t stream)
+cudaError_t launch_init_walkers(const SysParams *host_sys, int n_sys, cudaStream_t stream)
 {
-    (void)dev_sys;
-    for (int s = 0; s < n_sys; ++s) {
+    int dev = 0, sms = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    for (int s = 0; s < n_sys && e == cudaSuccess; ++s) {
         const SysParams &p = host_sys[s];
-        const size_t total = (size_t)p.n_walkers * (size_t)p.V;
-        const int threads = 256;
-        size_t blocks = (total + threads - 1) / threads;
-        if (blocks > 65536) blocks = 65536;
-        if (p.idx16)
-            fill_identity<uint16_t><<<(unsigned)blocks, threads, 0, stream>>>(p);
+        if (p.d == 2)
+            e = p.idx16 ? init_place<2, uint16_t>(p, optin, sms, stream) : init_place<2, uint32_t>(p, optin, sms, stream);
         else
-            fill_identity<uint32_t><<<(unsigned)blocks, threads, 0, stream>>>(p);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+            e = p.idx16 ? init_place<3, uint16_t>(p, optin, sms, stream) : init_place<3, uint32_t>(p, optin, sms, stream);
     }
-    return cudaSuccess;
-}
-
-cudaError_t launch_init_walkers(const SysParams *host_sys, const SysParams *dev_sys, int n_sys,
-                                cudaStream_t stream)
-{
-    for (int s = 0; s < n_sys; ++s) {
-        const int threads = 128;
-        const int blocks = (host_sys[s].n_walkers + threads - 1) / threads;
-        init_walkers_kernel<<<blocks, threads, 0, stream>>>(dev_sys, s);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return e;
 }
 
 cudaError_t walker_update_max_smem(int *bytes)

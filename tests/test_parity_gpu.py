@@ -715,3 +715,35 @@ def test_multi_commit_full_size_global_thresholds(wl_name):
             chain.run_walkers(d, L, N, seed, it, sweeps * N, -d * N, 0, T, S, occ, E, walkers=pick)
             for q, w in enumerate(pick):
                 _assert_walker_equal(mc, i, w, S[q], occ[q], E[q])
+
+
+# ------------------------------------------------- placement, list placements
+
+@pytest.mark.parametrize("desc", [
+    (2, 7, 48, 5, 0, 0, 1),          # one empty site: every step's targets collide
+    (3, 12, 1500, 9, 0, 0, 2),       # several chunks of targets, dense, ragged chunk and list
+    (2, 181, 1025, 3, 0, 0, 3),      # odd list length: walkers' lists off 16 bytes; 1024 + 1 targets
+    (3, 48, 2500, 2, 0, 0, 4),       # uint32 list too large for shared memory
+    (2, 1400, 1300, 2, 0, 0, 5),     # and the bitset too
+])
+def test_placement_batches_bit_exact(desc):
+    d, L, N, W, lo, hi, seed = desc
+    S, occ, E = _oracle_states(d, L, N, W, seed)
+    with m.Mucal([desc]) as mc:
+        for w in range(W):
+            _assert_walker_equal(mc, 0, w, S[w], occ[w], E[w])
+
+
+def test_histogram_rows_grow_with_the_launch_shape():
+    """Shapes with more blocks need more histogram rows; a captured iteration
+    does not keep the old ones."""
+    desc = (2, 16, 32, 64, 0, 0, 0)
+    S, occ, E = _oracle_states(2, 16, 32, 64, 0)
+    T = chain.thresholds(2, -64, 0, np.zeros(65))
+    with m.Mucal([desc]) as mc:
+        for it, (graph, wpb) in enumerate(((False, 64), (True, 64), (True, 1), (True, 64), (False, 2))):
+            mc.set_graph_mode(graph) if it in (1, 4) else None
+            mc.set_launch(kernel=m.MUCAL_KERNEL_THREAD, lanes_per_walker=1, walkers_per_block=wpb)
+            mc.run_iteration(3, it)
+            hist, _ = chain.run_walkers(2, 16, 32, 0, it, 96, -64, 0, T, S, occ, E)
+            np.testing.assert_array_equal(mc.histogram(0), hist.sum(axis=0))
