@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include "mucal.h"
+#include "mlp_adam.cuh"
 #include "mucal_internal.h"
 
 namespace {
@@ -388,28 +389,23 @@ mlp_dw2_kernel(const __nv_bfloat16 *__restrict__ dz2T, const __nv_bfloat16 *__re
         }
 }
 
-// Adam (Kingma and Ba) on the fp32 master parameters, then the bf16 copy.
-__global__ void mlp_adam_kernel(float *__restrict__ w, float *__restrict__ grad, float *__restrict__ m1,
-                                float *__restrict__ m2, __nv_bfloat16 *__restrict__ wq, int n, float lr,
-                                float beta1, float beta2, float eps, float c1, float c2)
+// Adam on all parameters from the summed gradient, which is cleared.
+__global__ void mlp_adam_kernel(mucal::AdamState st, float *__restrict__ grad, int n, float lr, float c1, float c2)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float gr = grad[i];
-    const float a = beta1 * m1[i] + (1.f - beta1) * gr;
-    const float b = beta2 * m2[i] + (1.f - beta2) * gr * gr;
-    m1[i] = a;
-    m2[i] = b;
-    const float v = w[i] - lr * (a / c1) / (sqrtf(b / c2) + eps);
-    w[i] = v;
-    wq[i] = __float2bfloat16_rn(v);
+    mucal::adam_step(st, i, grad[i], lr, c1, c2);
     grad[i] = 0.f;
 }
 
-__global__ void mlp_round_kernel(const float *__restrict__ w, __nv_bfloat16 *__restrict__ wq, int n)
+__global__ void mlp_round_kernel(mucal::AdamState st, int n)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) wq[i] = __float2bfloat16_rn(w[i]);
+    if (i >= n) return;
+    const __nv_bfloat16 q = __float2bfloat16_rn(st.w[i]);
+    st.wq[i] = q;
+    const int k = i - mucal::kMlpOffW2;
+    if (k >= 0 && k < H * H) st.w2t[(k % H) * H + k / H] = q;
 }
 
 // ---------------------------------------------------------------------------
@@ -420,7 +416,7 @@ struct Mlp {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     float *w = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr, *loss = nullptr;
-    __nv_bfloat16 *wq = nullptr;
+    __nv_bfloat16 *wq = nullptr, *w2t = nullptr;
     int64_t cap = 0;           // rows of the batch buffers (multiple of 256)
     float *X = nullptr, *t = nullptr, *y = nullptr;
     __nv_bfloat16 *h1T = nullptr, *dz2T = nullptr;
@@ -430,6 +426,7 @@ struct Mlp {
     bool use_tc = true;        // forward, gradients and training on tcgen05 (else mma.sync)
     int64_t step = 0;
     std::string err;
+    mucal::AdamState state() const { return {w, m1, m2, wq, w2t}; }
 };
 
 thread_local std::string g_mlp_err;
@@ -506,26 +503,34 @@ int check_tc(Mlp *m)
     return MUCAL_OK;
 }
 
+// The partial rows and the error flag of the tcgen05 training kernel.
+int ensure_tc(Mlp *m, int64_t B)
+{
+    int rc = ensure_err(m);
+    if (rc != MUCAL_OK) return rc;
+    const size_t need = mucal::mlp_train_tcgen05_partial_floats(B);
+    if (need > m->part_floats) {
+        MLP_TRY(m, cudaStreamSynchronize(m->stream));
+        cudaFree(m->part);
+        m->part = nullptr;
+        m->part_floats = 0;
+        MLP_TRY(m, cudaMalloc(&m->part, need * sizeof(float)));
+        m->part_floats = need;
+    }
+    return MUCAL_OK;
+}
+
 int enqueue_grad(Mlp *m, int64_t B)
 {
     const int blocks = (int)((B + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK);
-    MLP_TRY(m, cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
     if (m->use_tc) {
-        int rc = ensure_err(m);
+        int rc = ensure_tc(m, B);
         if (rc != MUCAL_OK) return rc;
-        const size_t need = mucal::mlp_train_tcgen05_partial_floats(B);
-        if (need > m->part_floats) {
-            MLP_TRY(m, cudaStreamSynchronize(m->stream));
-            cudaFree(m->part);
-            m->part = nullptr;
-            m->part_floats = 0;
-            MLP_TRY(m, cudaMalloc(&m->part, need * sizeof(float)));
-            m->part_floats = need;
-        }
-        MLP_TRY(m, mucal::mlp_train_tcgen05(m->wq, m->X, m->t, B, m->part, m->grad, m->loss,
+        MLP_TRY(m, mucal::mlp_train_tcgen05(m->state(), m->X, m->t, B, m->part, m->grad, m->loss,
                                             m->d_err, m->stream));
         return MUCAL_OK;
     }
+    MLP_TRY(m, cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
     mlp_rows_kernel<true><<<blocks, WARPS * 32, rows_smem(), m->stream>>>(
         m->wq, m->X, m->t, m->y, B, 1.0f / (float)B, m->h1T, m->dz2T, m->cap, m->grad, m->loss);
     MLP_TRY(m, cudaGetLastError());
@@ -560,7 +565,7 @@ int mucal_mlp_create(void **out, const float *params, int64_t n, void *cuda_stre
     Mlp *m = new Mlp();
     auto bail = [&](int code) {
         g_mlp_err = m->err;
-        cudaFree(m->w); cudaFree(m->grad); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->wq);
+        cudaFree(m->w); cudaFree(m->grad); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->wq); cudaFree(m->w2t);
         cudaFree(m->loss);
         if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
         delete m;
@@ -576,7 +581,8 @@ int mucal_mlp_create(void **out, const float *params, int64_t n, void *cuda_stre
     }
     if (cudaMalloc(&m->w, NPARAM * 4) != cudaSuccess || cudaMalloc(&m->grad, NPARAM * 4) != cudaSuccess ||
         cudaMalloc(&m->m1, NPARAM * 4) != cudaSuccess || cudaMalloc(&m->m2, NPARAM * 4) != cudaSuccess ||
-        cudaMalloc(&m->wq, NPARAM * 2) != cudaSuccess || cudaMalloc(&m->loss, 4) != cudaSuccess)
+        cudaMalloc(&m->wq, NPARAM * 2) != cudaSuccess || cudaMalloc(&m->w2t, H * H * 2) != cudaSuccess ||
+        cudaMalloc(&m->loss, 4) != cudaSuccess)
         return bail(mfail(m, MUCAL_ERR_OOM, "cudaMalloc failed"));
     if (cudaFuncSetAttribute(mlp_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)rows_smem()) != cudaSuccess ||
@@ -588,7 +594,7 @@ int mucal_mlp_create(void **out, const float *params, int64_t n, void *cuda_stre
         cudaMemsetAsync(m->m1, 0, NPARAM * 4, m->stream) != cudaSuccess ||
         cudaMemsetAsync(m->m2, 0, NPARAM * 4, m->stream) != cudaSuccess)
         return bail(mfail(m, MUCAL_ERR_CUDA, "parameter upload failed"));
-    mlp_round_kernel<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(m->w, m->wq, NPARAM);
+    mlp_round_kernel<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(m->state(), NPARAM);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(m->stream) != cudaSuccess)
         return bail(mfail(m, MUCAL_ERR_CUDA, "parameter rounding failed"));
     *out = m;
@@ -601,7 +607,7 @@ void mucal_mlp_destroy(void *mlp)
     if (!m) return;
     cudaSetDevice(m->device);
     cudaStreamSynchronize(m->stream);
-    cudaFree(m->w); cudaFree(m->grad); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->wq);
+    cudaFree(m->w); cudaFree(m->grad); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->wq); cudaFree(m->w2t);
     cudaFree(m->loss); cudaFree(m->X); cudaFree(m->t); cudaFree(m->y); cudaFree(m->h1T);
     cudaFree(m->dz2T); cudaFree(m->part);
     cudaFree(m->d_err);
@@ -697,15 +703,24 @@ int mucal_mlp_train(void *mlp, const float *X, const float *t, int64_t B, int32_
     int rc = upload_batch(m, X, t, B);
     if (rc != MUCAL_OK) return rc;
     MLP_TRY(m, cudaMemsetAsync(m->grad, 0, NPARAM * 4, m->stream));
-    const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
-    for (int s = 0; s < steps; ++s) {
-        rc = enqueue_grad(m, B);
+    if (m->use_tc) {
+        rc = ensure_tc(m, B);
         if (rc != MUCAL_OK) return rc;
+    }
+    for (int s = 0; s < steps; ++s) {
+        if (!m->use_tc) {
+            rc = enqueue_grad(m, B);
+            if (rc != MUCAL_OK) return rc;
+        }
         m->step += 1;
-        const float c1 = 1.f - std::pow(beta1, (float)m->step);
-        const float c2 = 1.f - std::pow(beta2, (float)m->step);
-        mlp_adam_kernel<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(
-            m->w, m->grad, m->m1, m->m2, m->wq, NPARAM, lr, beta1, beta2, eps, c1, c2);
+        const float c1 = 1.f - std::pow(mucal::kAdamBeta1, (float)m->step);
+        const float c2 = 1.f - std::pow(mucal::kAdamBeta2, (float)m->step);
+        if (m->use_tc) {
+            MLP_TRY(m, mucal::mlp_train_step_tcgen05(m->state(), m->X, m->t, B, m->part, m->loss, m->d_err, lr,
+                                                     c1, c2, m->stream));
+            continue;
+        }
+        mlp_adam_kernel<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(m->state(), m->grad, NPARAM, lr, c1, c2);
         MLP_TRY(m, cudaGetLastError());
     }
     if (loss_out) MLP_TRY(m, cudaMemcpyAsync(loss_out, m->loss, 4, cudaMemcpyDeviceToHost, m->stream));

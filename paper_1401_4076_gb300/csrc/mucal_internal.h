@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 namespace mucal {
@@ -166,13 +167,24 @@ cudaError_t launch_droplets(const SysParams &p, const DropletOut &o, const Dropl
 // non-zero if a tensor-core wait ran out.
 cudaError_t mlp_forward_tcgen05(const void *wq, const float *X, float *y, int64_t B, int *err,
                                 cudaStream_t stream);
+// The seeding network's parameters (fp32 master copy, Adam moments, the bf16
+// copy that the kernels compute with and the transposed bf16 W2).
+constexpr int kMlpH = 128, kMlpOffW2 = kMlpH * 5;
+struct AdamState {
+    float *w, *m1, *m2;
+    __nv_bfloat16 *wq, *w2t;
+};
 // Gradients of the mean squared error against target[B] written to grad
 // (fp32[17281]) and the loss to *loss, every contraction on tcgen05.  part
 // holds mlp_train_tcgen05_partial_floats(B) floats: one row per CTA, summed
 // in CTA order, so the result does not depend on the CTAs' finishing order.
 size_t mlp_train_tcgen05_partial_floats(int64_t B);
-cudaError_t mlp_train_tcgen05(const void *wq, const float *X, const float *target, int64_t B,
+cudaError_t mlp_train_tcgen05(const AdamState &st, const float *X, const float *target, int64_t B,
                               float *part, float *grad, float *loss, int *err, cudaStream_t stream);
+// The same gradients and the Adam step with them (bias corrections c1, c2).
+cudaError_t mlp_train_step_tcgen05(const AdamState &st, const float *X, const float *target, int64_t B,
+                                   float *part, float *loss, int *err, float lr, float c1, float c2,
+                                   cudaStream_t stream);
 
 // Error message of calls that have no context (mucal_host.cu).
 void set_init_error(const char *msg);
