@@ -38,7 +38,7 @@ struct System {
     bool target_default = true;
     uint32_t *thr_pinned = nullptr; // staging buffer of the threshold upload
     size_t thr_count = 0;
-    size_t hist_cap = 0;            // histogram rows allocated
+    size_t h_off = 0;               // its place in the context's summed histograms
     uint64_t last_attempts = 0;
     std::vector<double> lnW_run;    // the weights of the last iteration's thresholds
     unsigned long long *drop_acc = nullptr;  // device [3][n_bins] droplet accumulators
@@ -68,6 +68,14 @@ struct Context {
     bool measured = false;
     bool tunnel = false;                 // walker kernels with tunnelling bookkeeping
     int *d_next_item = nullptr;          // work-item counter of persistent launches
+    // all systems' summed histograms and, behind them, the walker kernels' error
+    // flag: one block, one clear and one copy per iteration for all systems
+    unsigned long long *d_H = nullptr, *h_H = nullptr;   // device, pinned host
+    size_t h_words = 0;                  // words of the histograms
+    unsigned long long *d_hist = nullptr;    // all systems' histogram rows
+    size_t hist_words = 0, hist_cap = 0;     // words in use, words allocated
+    mucal::ReduceWork *d_reduce = nullptr;   // blocks of the histogram sum
+    int n_reduce = 0;
     unsigned int *d_walk_err = nullptr;  // set by a walker kernel whose bounded wait ran out
     // CUDA-graph mode: one graph per (sweeps, launch shape, flavour, grid)
     bool graph_mode = false;
@@ -82,7 +90,7 @@ struct Context {
     uint32_t *d_xthr = nullptr;          // replica-exchange thresholds, [pairs][2 n_bins - 1]
     uint32_t *xthr_pinned = nullptr;     // their host staging buffer
     size_t xthr_words = 0;
-    unsigned long long *d_xacc = nullptr;  // accepted exchanges per pair
+    unsigned long long *d_xacc = nullptr, *xacc_pinned = nullptr;  // accepted exchanges per pair
     std::string err;
 };
 
@@ -321,11 +329,9 @@ void free_system(System &s)
     cudaFree(s.p.bits);
     cudaFree(s.p.S);
     cudaFree(s.p.E);
-    cudaFree(s.p.hist);
     cudaFree((void *)s.p.thr);
     cudaFree((void *)s.p.thrT);
     cudaFree(s.p.accepts);
-    cudaFree(s.p.H);
     if (s.thr_pinned) cudaFreeHost(s.thr_pinned);
     cudaFree(s.drop_acc);
     cudaFree(s.drop_last);
@@ -350,8 +356,12 @@ void destroy_context(Context *c)
     cudaFree(c->d_xthr);
     cudaFree(c->d_xacc);
     if (c->xthr_pinned) cudaFreeHost(c->xthr_pinned);
+    if (c->xacc_pinned) cudaFreeHost(c->xacc_pinned);
     cudaFree(c->d_next_item);
-    cudaFree(c->d_walk_err);
+    cudaFree(c->d_H);
+    if (c->h_H) cudaFreeHost(c->h_H);
+    cudaFree(c->d_hist);
+    cudaFree(c->d_reduce);
     if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
     if (c->graph) cudaGraphDestroy(c->graph);
     if (c->ev_it0) cudaEventDestroy(c->ev_it0);
@@ -402,7 +412,6 @@ int build_work(Context *c, const LaunchShape &sh)
             ++rows;
             work.push_back(bw);
         }
-        // blocks never outnumber walkers, so the per-walker allocation holds them
         rows_of[s] = per_walker ? p.n_walkers : rows;
     }
     std::stable_sort(work.begin(), work.end(), [&](const BlockWork &a, const BlockWork &b) {
@@ -410,27 +419,41 @@ int build_work(Context *c, const LaunchShape &sh)
         const double cb = (double)c->sys[b.sys].p.N * c->sys[b.sys].p.d;
         return ca > cb;
     });
+    std::vector<mucal::ReduceWork> reduce;
+    std::vector<size_t> off(c->sys.size(), 0);
+    size_t words = 0;
+    for (int s = 0; s < (int)c->sys.size(); ++s) {
+        const int bins = c->sys[s].p.n_bins;
+        off[s] = words;
+        words += (size_t)rows_of[s] * (size_t)bins;
+        for (int r = 0; r < rows_of[s]; r += mucal::kReduceRows)
+            for (int b = 0; b < bins; b += mucal::kReduceBins) reduce.push_back({s, b, r});
+    }
     // build the new tables completely before replacing the old ones, so that
     // a failure leaves the previous launch shape usable
     BlockWork *d_work = nullptr;
-    cudaError_t e = cudaMalloc(&d_work, std::max<size_t>(1, work.size()) * sizeof(BlockWork));
+    mucal::ReduceWork *d_reduce = nullptr;
+    unsigned long long *d_hist = nullptr;
+    cudaError_t e = cudaMalloc(&d_work, work.size() * sizeof(BlockWork));
+    if (e == cudaSuccess) e = cudaMalloc(&d_reduce, reduce.size() * sizeof(mucal::ReduceWork));
     if (e == cudaSuccess)
         e = cudaMemcpy(d_work, work.data(), work.size() * sizeof(BlockWork), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(d_reduce, reduce.data(), reduce.size() * sizeof(mucal::ReduceWork),
+                       cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && words > c->hist_cap) e = cudaMalloc(&d_hist, words * 8);
     std::vector<SysParams> hp(c->sys.size());
-    std::vector<void *> grown(c->sys.size(), nullptr);
     for (size_t i = 0; i < c->sys.size(); ++i) {
         hp[i] = c->sys[i].p;
         hp[i].hist_rows = rows_of[i];
-        if (e == cudaSuccess && (size_t)rows_of[i] > c->sys[i].hist_cap) {
-            e = cudaMalloc(&grown[i], (size_t)rows_of[i] * (size_t)hp[i].n_bins * 8);
-            hp[i].hist = static_cast<unsigned long long *>(grown[i]);
-        }
+        hp[i].hist = (d_hist ? d_hist : c->d_hist) + off[i];
     }
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_sys, hp.data(), hp.size() * sizeof(SysParams), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(d_work);
-        for (void *q : grown) cudaFree(q);
+        cudaFree(d_reduce);
+        cudaFree(d_hist);
         // restore the device table of the current shape
         std::vector<SysParams> cur(c->sys.size());
         for (size_t i = 0; i < c->sys.size(); ++i) cur[i] = c->sys[i].p;
@@ -438,16 +461,22 @@ int build_work(Context *c, const LaunchShape &sh)
         return fail(c, e == cudaErrorMemoryAllocation ? MUCAL_ERR_OOM : MUCAL_ERR_CUDA,
                     "launch table upload failed: %s", cudaGetErrorString(e));
     }
+    drop_graph(c);               // a captured iteration holds the old tables and rows
     cudaFree(c->d_work);
+    cudaFree(c->d_reduce);
     c->d_work = d_work;
     c->n_blocks = (int)work.size();
+    c->d_reduce = d_reduce;
+    c->n_reduce = (int)reduce.size();
+    if (d_hist) {
+        cudaFree(c->d_hist);
+        c->d_hist = d_hist;
+        c->hist_cap = words;
+    }
+    c->hist_words = words;
     for (size_t i = 0; i < c->sys.size(); ++i) {
         c->sys[i].p.hist_rows = rows_of[i];
-        if (!grown[i]) continue;
-        drop_graph(c);               // a captured iteration holds the old rows
-        cudaFree(c->sys[i].p.hist);
         c->sys[i].p.hist = hp[i].hist;
-        c->sys[i].hist_cap = (size_t)rows_of[i];
     }
     return MUCAL_OK;
 }
@@ -656,21 +685,25 @@ int check_sys(Context *c, int32_t s)
     return MUCAL_OK;
 }
 
+// Every system's summed histogram to the host, with the error flag behind
+// them, by one copy into pinned memory (a copy per system and one for the
+// flag, both pageable, cost an 8-system tempering round 0.13 ms).
 int fetch_histogram(Context *c, System &s)
 {
     if (!c->ran) return fail(c, MUCAL_ERR_NOT_READY, "no iteration has been run");
-    if (!s.hist_on_host) {
-        unsigned int err = 0;
-        CUDA_TRY(c, cudaMemcpyAsync(s.H.data(), s.p.H, s.H.size() * sizeof(int64_t),
-                                    cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(c, cudaMemcpyAsync(&err, c->d_walk_err, sizeof err, cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        if (err) {
-            CUDA_TRY(c, cudaMemsetAsync(c->d_walk_err, 0, sizeof err, c->stream));
-            return fail(c, MUCAL_ERR_STATE, "a walker kernel's wait for its threshold rows ran out "
-                                            "(flag %u); the iteration's results are not valid", err);
-        }
-        s.hist_on_host = true;
+    if (s.hist_on_host) return MUCAL_OK;
+    CUDA_TRY(c, cudaMemcpyAsync(c->h_H, c->d_H, (c->h_words + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    const unsigned int err = (unsigned int)c->h_H[c->h_words];
+    if (err) {
+        CUDA_TRY(c, cudaMemsetAsync(c->d_walk_err, 0, 8, c->stream));
+        return fail(c, MUCAL_ERR_STATE, "a walker kernel's wait for its threshold rows ran out "
+                                        "(flag %u); the iteration's results are not valid", err);
+    }
+    for (auto &q : c->sys) {
+        if (q.hist_on_host) continue;
+        std::memcpy(q.H.data(), c->h_H + q.h_off, q.H.size() * sizeof(int64_t));
+        q.hist_on_host = true;
     }
     return MUCAL_OK;
 }
@@ -700,19 +733,14 @@ int reset_tunnel(Context *c, const System &s)
 int enqueue_iteration(Context *c, uint64_t sweeps, uint32_t iteration, int grid, bool events)
 {
     if (events) CUDA_TRY(c, cudaEventRecord(c->ev_it0, c->stream));
-    for (auto &s : c->sys) {
-        CUDA_TRY(c, cudaMemsetAsync(s.p.hist, 0, (size_t)s.p.hist_rows * (size_t)s.p.n_bins * 8,
-                                    c->stream));
-        CUDA_TRY(c, cudaMemsetAsync(s.p.H, 0, (size_t)s.p.n_bins * 8, c->stream));
-    }
+    CUDA_TRY(c, cudaMemsetAsync(c->d_hist, 0, c->hist_words * 8, c->stream));
+    CUDA_TRY(c, cudaMemsetAsync(c->d_H, 0, c->h_words * 8, c->stream));
     if (c->shape.persistent) CUDA_TRY(c, cudaMemsetAsync(c->d_next_item, 0, sizeof(int), c->stream));
     if (events) CUDA_TRY(c, cudaEventRecord(c->ev_k0, c->stream));
     CUDA_TRY(c, mucal::launch_walker_update(c->d_sys, c->d_work, c->n_blocks, c->shape, sweeps,
                                             iteration, c->tunnel, grid, c->d_next_item, c->stream));
     if (events) CUDA_TRY(c, cudaEventRecord(c->ev_k1, c->stream));
-    std::vector<SysParams> hp(c->sys.size());
-    for (size_t i = 0; i < c->sys.size(); ++i) hp[i] = c->sys[i].p;
-    CUDA_TRY(c, mucal::launch_hist_reduce(hp.data(), c->d_sys, (int)hp.size(), c->stream));
+    CUDA_TRY(c, mucal::launch_hist_reduce(c->d_sys, c->d_reduce, c->n_reduce, c->stream));
     if (events) CUDA_TRY(c, cudaEventRecord(c->ev_it1, c->stream));
     return MUCAL_OK;
 }
@@ -882,7 +910,6 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
         ALLOC(E, nw * sizeof(int32_t));
         ALLOC(thr, (size_t)p.n_bins * p.tstride * sizeof(uint32_t));
         ALLOC(accepts, nw * sizeof(unsigned long long));
-        ALLOC(H, (size_t)p.n_bins * sizeof(unsigned long long));
         ALLOC(tun_state, nw * sizeof(uint8_t));
         ALLOC(tun_count, nw * sizeof(uint32_t));
 #undef ALLOC
@@ -912,7 +939,6 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
             cudaMemsetAsync(s.drop_last, 0, nw * sizeof(int32_t), c->stream) != cudaSuccess)
             return bail(fail(nullptr, MUCAL_ERR_CUDA, "memset failed"));
         if (cudaMemsetAsync(p.bits, 0, nw * p.words * sizeof(uint32_t), c->stream) != cudaSuccess ||
-            cudaMemsetAsync(p.H, 0, (size_t)p.n_bins * 8, c->stream) != cudaSuccess ||
             cudaMemsetAsync(p.accepts, 0, nw * 8, c->stream) != cudaSuccess ||
             cudaMemsetAsync(p.tun_state, 0, nw, c->stream) != cudaSuccess ||
             cudaMemsetAsync(p.tun_count, 0, nw * 4, c->stream) != cudaSuccess)
@@ -923,10 +949,19 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
     for (auto &s : c->sys) s.p.prefetch = lists > kListsInL2 ? 1 : 0;
     if (cudaMalloc(&c->d_next_item, sizeof(int)) != cudaSuccess)
         return bail(fail(nullptr, MUCAL_ERR_OOM, "cudaMalloc of the work-item counter failed"));
-    if (cudaMalloc(&c->d_walk_err, sizeof(unsigned int)) != cudaSuccess ||
-        cudaMemsetAsync(c->d_walk_err, 0, sizeof(unsigned int), c->stream) != cudaSuccess)
-        return bail(fail(nullptr, MUCAL_ERR_OOM, "cudaMalloc of the walker error flag failed"));
-    for (auto &s : c->sys) s.p.err = c->d_walk_err;
+    for (auto &s : c->sys) {
+        s.h_off = c->h_words;
+        c->h_words += (size_t)s.p.n_bins;
+    }
+    if (cudaMalloc(&c->d_H, (c->h_words + 1) * 8) != cudaSuccess ||
+        cudaMallocHost(&c->h_H, (c->h_words + 1) * 8) != cudaSuccess ||
+        cudaMemsetAsync(c->d_H, 0, (c->h_words + 1) * 8, c->stream) != cudaSuccess)
+        return bail(fail(nullptr, MUCAL_ERR_OOM, "allocation of the summed histograms failed"));
+    c->d_walk_err = reinterpret_cast<unsigned int *>(c->d_H + c->h_words);
+    for (auto &s : c->sys) {
+        s.p.H = c->d_H + s.h_off;
+        s.p.err = c->d_walk_err;
+    }
     if (cudaMalloc(&c->d_drop_err, sizeof(int)) != cudaSuccess ||
         cudaMemsetAsync(c->d_drop_err, 0, sizeof(int), c->stream) != cudaSuccess)
         return bail(fail(nullptr, MUCAL_ERR_OOM, "cudaMalloc of the droplet error flag failed"));
@@ -1406,13 +1441,16 @@ int mucal_replica_exchange(void *ctx, const double *beta, int32_t n_sys, uint32_
         cudaFree(c->d_xthr);
         cudaFree(c->d_xacc);
         if (c->xthr_pinned) cudaFreeHost(c->xthr_pinned);
+        if (c->xacc_pinned) cudaFreeHost(c->xacc_pinned);
         c->d_xthr = nullptr;
         c->d_xacc = nullptr;
         c->xthr_pinned = nullptr;
+        c->xacc_pinned = nullptr;
         c->xthr_words = 0;
         CUDA_TRY(c, cudaMalloc(&c->d_xthr, words * sizeof(uint32_t)));
         CUDA_TRY(c, cudaMalloc(&c->d_xacc, (size_t)pairs * sizeof(unsigned long long)));
         CUDA_TRY(c, cudaMallocHost(&c->xthr_pinned, words * sizeof(uint32_t)));
+        CUDA_TRY(c, cudaMallocHost(&c->xacc_pinned, (size_t)pairs * sizeof(unsigned long long)));
         c->xthr_words = words;
     }
     // the staging buffer may still feed the previous exchange's upload
@@ -1436,9 +1474,10 @@ int mucal_replica_exchange(void *ctx, const double *beta, int32_t n_sys, uint32_
     CUDA_TRY(c, mucal::launch_exchange(c->d_sys, n_sys, p0.n_walkers, parity, round, c->d_xthr, width,
                                        c->d_xacc, c->stream));
     if (accepted) {
-        CUDA_TRY(c, cudaMemcpyAsync(accepted, c->d_xacc, (size_t)pairs * 8, cudaMemcpyDeviceToHost,
+        CUDA_TRY(c, cudaMemcpyAsync(c->xacc_pinned, c->d_xacc, (size_t)pairs * 8, cudaMemcpyDeviceToHost,
                                     c->stream));
         CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+        std::memcpy(accepted, c->xacc_pinned, (size_t)pairs * 8);
     }
     return MUCAL_OK;
 }

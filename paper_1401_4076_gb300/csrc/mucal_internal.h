@@ -64,6 +64,15 @@ struct BlockWork {
     int32_t hist_row;   // this block's histogram row when rows are per block, else -1
 };
 
+// One block of the histogram sum: kReduceBins bins from bin0 on of kReduceRows
+// rows from row0 on of system sys.
+constexpr int kReduceBins = 256, kReduceRows = 16;
+struct ReduceWork {
+    int32_t sys;
+    int32_t bin0;
+    int32_t row0;
+};
+
 // Walker-update kernels of one (tunnelling, persistent) flavour: the thread
 // kernel in its shared-memory variants, the group kernel with the bitsets in
 // shared or global memory and the thresholds in global memory, in shared
@@ -132,7 +141,7 @@ size_t thr_smem_words(const SysParams &p);
 size_t thr_window_bytes(const SysParams &p);
 // Shared-memory bytes of one walker's neighbour-count field (field kernel).
 size_t field_smem_bytes(const SysParams &p);
-cudaError_t launch_hist_reduce(const SysParams *host_sys, const SysParams *dev_sys, int n_sys,
+cudaError_t launch_hist_reduce(const SysParams *dev_sys, const ReduceWork *dev_work, int n_items,
                                cudaStream_t stream);
 cudaError_t walker_update_max_smem(int *bytes);
 // Rewrite the dE-major copy of system p's threshold table from p.thr.

@@ -190,22 +190,38 @@ cudaError_t init_place(const SysParams &p, int optin, int sms, cudaStream_t stre
 }
 
 // ---------------------------------------------------------------------------
-// H(E) = sum_j H_j(E) (Eq. 2).  Block (x: 256 bins, y: a chunk of walkers);
-// each thread sums its bin over the chunk (coalesced across the bins) and
-// adds the partial sum to H with one 64-bit atomic.
+// H(E) = sum_j H_j(E) (Eq. 2).  A block sums 256 bins of a chunk of rows
+// (coalesced across the bins), each thread its bin's rows with all loads in
+// flight, and adds the partial sum to H with one 64-bit atomic.  All systems'
+// blocks are one launch (ReduceWork): bound by the latency of one chunk, so a
+// launch per system made a context of 27 systems wait 27 times (0.10 ms an
+// iteration) and chunks of 64 rows left most SMs idle (2D L = 64: 12 blocks;
+// 40 now).
 // ---------------------------------------------------------------------------
-constexpr int kReduceWalkers = 64;
-
-__global__ void hist_reduce_kernel(SysParams p)
+__device__ __forceinline__ void hist_reduce_block(const SysParams &p, int bin0, int row0)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = bin0 + (int)threadIdx.x;
     if (b >= p.n_bins) return;
-    const int w0 = blockIdx.y * kReduceWalkers;
-    const int w1 = min(w0 + kReduceWalkers, p.hist_rows);
+    const unsigned long long *h = p.hist + (size_t)row0 * (size_t)p.n_bins + b;
+    const int rows = min(kReduceRows, p.hist_rows - row0);
     unsigned long long sum = 0;
-    const unsigned long long *h = p.hist + (size_t)w0 * (size_t)p.n_bins + b;
-    for (int w = w0; w < w1; ++w, h += p.n_bins) sum += *h;
+#pragma unroll
+    for (int r = 0; r < kReduceRows; ++r) sum += r < rows ? h[(size_t)r * (size_t)p.n_bins] : 0ull;
     if (sum) atomicAdd(p.H + b, sum);
+}
+
+__global__ void __launch_bounds__(kReduceBins)
+hist_reduce_kernel(const SysParams *__restrict__ sys, const ReduceWork *__restrict__ work)
+{
+    const ReduceWork wk = work[blockIdx.x];
+    hist_reduce_block(sys[wk.sys], wk.bin0, wk.row0);
+}
+
+// The same for one system given by value (x: bins, y: rows).
+__global__ void __launch_bounds__(kReduceBins)
+hist_reduce_one_kernel(SysParams p)
+{
+    hist_reduce_block(p, (int)blockIdx.x * kReduceBins, (int)blockIdx.y * kReduceRows);
 }
 
 // The dE-major copy of a threshold table: entry (b, j) to row j, word
@@ -423,18 +439,11 @@ size_t field_smem_bytes(const SysParams &p) { return field_bytes(p); }
 
 size_t thr_window_bytes(const SysParams &p) { return window_bytes(p); }
 
-cudaError_t launch_hist_reduce(const SysParams *host_sys, const SysParams *dev_sys, int n_sys,
+cudaError_t launch_hist_reduce(const SysParams *dev_sys, const ReduceWork *dev_work, int n_items,
                                cudaStream_t stream)
 {
-    (void)dev_sys;
-    for (int s = 0; s < n_sys; ++s) {
-        const SysParams &p = host_sys[s];
-        dim3 grid((p.n_bins + 255) / 256, (p.hist_rows + kReduceWalkers - 1) / kReduceWalkers);
-        hist_reduce_kernel<<<grid, 256, 0, stream>>>(p);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    hist_reduce_kernel<<<n_items, kReduceBins, 0, stream>>>(dev_sys, dev_work);
+    return cudaGetLastError();
 }
 
 }  // namespace mucal
@@ -686,8 +695,8 @@ extern "C" int mucal_run_walkers_noalloc(const mucal_system_desc *sys, int64_t s
         ce = cudaGetLastError();
     }
     if (ce == cudaSuccess) {
-        dim3 grid((p.n_bins + 255) / 256, (p.hist_rows + kReduceWalkers - 1) / kReduceWalkers);
-        hist_reduce_kernel<<<grid, 256, 0, st>>>(p);
+        dim3 grid((p.n_bins + kReduceBins - 1) / kReduceBins, (p.hist_rows + kReduceRows - 1) / kReduceRows);
+        hist_reduce_one_kernel<<<grid, kReduceBins, 0, st>>>(p);
         ce = cudaGetLastError();
     }
     unsigned long long bad = 0;
