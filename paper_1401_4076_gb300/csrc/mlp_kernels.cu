@@ -420,7 +420,9 @@ struct Mlp {
     int64_t cap = 0;           // rows of the batch buffers (multiple of 256)
     float *X = nullptr, *t = nullptr, *y = nullptr;
     __nv_bfloat16 *h1T = nullptr, *dz2T = nullptr;
-    int *d_err = nullptr;      // error flag of the tcgen05 kernels
+    // error flag of the tcgen05 kernels, in mapped host memory: no copy per call
+    volatile int *h_err = nullptr;
+    int *d_err = nullptr;      // its device address
     float *part = nullptr;     // per-CTA gradient rows of the tcgen05 training kernel
     size_t part_floats = 0;
     bool use_tc = true;        // forward, gradients and training on tcgen05 (else mma.sync)
@@ -462,15 +464,18 @@ int ensure_capacity(Mlp *m, int64_t B)
     return MUCAL_OK;
 }
 
-int upload_batch(Mlp *m, const float *X, const float *t, int64_t B)
+// (the tcgen05 kernels leave out rows past B by themselves; the mma.sync ones
+// need the padding cleared)
+int upload_batch(Mlp *m, const float *X, const float *t, int64_t B, bool tc)
 {
     int rc = ensure_capacity(m, B);
     if (rc != MUCAL_OK) return rc;
-    MLP_TRY(m, cudaMemsetAsync(m->X, 0, m->cap * 4 * sizeof(float), m->stream));
+    if (!tc) MLP_TRY(m, cudaMemsetAsync(m->X, 0, m->cap * 4 * sizeof(float), m->stream));
     MLP_TRY(m, cudaMemcpyAsync(m->X, X, B * 4 * sizeof(float), cudaMemcpyHostToDevice, m->stream));
     if (t) {
-        MLP_TRY(m, cudaMemsetAsync(m->t, 0, m->cap * sizeof(float), m->stream));
+        if (!tc) MLP_TRY(m, cudaMemsetAsync(m->t, 0, m->cap * sizeof(float), m->stream));
         MLP_TRY(m, cudaMemcpyAsync(m->t, t, B * sizeof(float), cudaMemcpyHostToDevice, m->stream));
+        if (tc) return MUCAL_OK;
         // rows past B contribute nothing: their dz2 is zero
         MLP_TRY(m, cudaMemsetAsync(m->h1T, 0, (size_t)H * m->cap * sizeof(__nv_bfloat16), m->stream));
         MLP_TRY(m, cudaMemsetAsync(m->dz2T, 0, (size_t)H * m->cap * sizeof(__nv_bfloat16), m->stream));
@@ -482,22 +487,23 @@ size_t rows_smem() { return sizeof(MlpShared); }
 
 int ensure_err(Mlp *m)
 {
-    if (!m->d_err) {
-        MLP_TRY(m, cudaMalloc(&m->d_err, sizeof(int)));
-        MLP_TRY(m, cudaMemsetAsync(m->d_err, 0, sizeof(int), m->stream));
+    if (!m->h_err) {
+        void *q = nullptr;
+        MLP_TRY(m, cudaHostAlloc(&q, sizeof(int), cudaHostAllocMapped));
+        m->h_err = static_cast<volatile int *>(q);
+        *m->h_err = 0;
+        MLP_TRY(m, cudaHostGetDevicePointer(&q, q, 0));
+        m->d_err = static_cast<int *>(q);
     }
     return MUCAL_OK;
 }
 
-// Read and clear the tcgen05 error flag (waits for the stream).
+// Wait for the stream, then read and clear the tcgen05 error flag.
 int check_tc(Mlp *m)
 {
-    if (!m->d_err) return MUCAL_OK;
-    int flag = 0;
-    MLP_TRY(m, cudaMemcpyAsync(&flag, m->d_err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
     MLP_TRY(m, cudaStreamSynchronize(m->stream));
-    if (flag) {
-        MLP_TRY(m, cudaMemset(m->d_err, 0, sizeof(int)));
+    if (m->h_err && *m->h_err) {
+        *m->h_err = 0;
         return mfail(m, MUCAL_ERR_STATE, "tcgen05 kernel: a tensor-core wait ran out");
     }
     return MUCAL_OK;
@@ -610,7 +616,7 @@ void mucal_mlp_destroy(void *mlp)
     cudaFree(m->w); cudaFree(m->grad); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->wq); cudaFree(m->w2t);
     cudaFree(m->loss); cudaFree(m->X); cudaFree(m->t); cudaFree(m->y); cudaFree(m->h1T);
     cudaFree(m->dz2T); cudaFree(m->part);
-    cudaFree(m->d_err);
+    if (m->h_err) cudaFreeHost(const_cast<int *>(m->h_err));
     if (m->own_stream) cudaStreamDestroy(m->stream);
     delete m;
 }
@@ -651,7 +657,7 @@ int mucal_mlp_forward(void *mlp, const float *X, int64_t B, float *y)
     if (m && m->use_tc) return mucal_mlp_forward_tcgen05(mlp, X, B, y);
     if (!m || !X || !y || B <= 0) return mfail(m, MUCAL_ERR_INVALID_ARG, "bad forward arguments");
     MLP_TRY(m, cudaSetDevice(m->device));
-    int rc = upload_batch(m, X, nullptr, B);
+    int rc = upload_batch(m, X, nullptr, B, false);
     if (rc != MUCAL_OK) return rc;
     const int blocks = (int)((B + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK);
     mlp_rows_kernel<false><<<blocks, WARPS * 32, rows_smem(), m->stream>>>(
@@ -667,7 +673,7 @@ int mucal_mlp_forward_tcgen05(void *mlp, const float *X, int64_t B, float *y)
     Mlp *m = static_cast<Mlp *>(mlp);
     if (!m || !X || !y || B <= 0) return mfail(m, MUCAL_ERR_INVALID_ARG, "bad forward arguments");
     MLP_TRY(m, cudaSetDevice(m->device));
-    int rc = upload_batch(m, X, nullptr, B);
+    int rc = upload_batch(m, X, nullptr, B, true);
     if (rc != MUCAL_OK) return rc;
     rc = ensure_err(m);
     if (rc != MUCAL_OK) return rc;
@@ -681,7 +687,7 @@ int mucal_mlp_gradients(void *mlp, const float *X, const float *t, int64_t B, fl
     Mlp *m = static_cast<Mlp *>(mlp);
     if (!m || !X || !t || B <= 0) return mfail(m, MUCAL_ERR_INVALID_ARG, "bad gradient arguments");
     MLP_TRY(m, cudaSetDevice(m->device));
-    int rc = upload_batch(m, X, t, B);
+    int rc = upload_batch(m, X, t, B, m->use_tc);
     if (rc != MUCAL_OK) return rc;
     MLP_TRY(m, cudaMemsetAsync(m->grad, 0, NPARAM * 4, m->stream));
     rc = enqueue_grad(m, B);
@@ -689,7 +695,6 @@ int mucal_mlp_gradients(void *mlp, const float *X, const float *t, int64_t B, fl
     if (grad) MLP_TRY(m, cudaMemcpyAsync(grad, m->grad, NPARAM * 4, cudaMemcpyDeviceToHost, m->stream));
     if (loss) MLP_TRY(m, cudaMemcpyAsync(loss, m->loss, 4, cudaMemcpyDeviceToHost, m->stream));
     MLP_TRY(m, cudaMemsetAsync(m->grad, 0, NPARAM * 4, m->stream));
-    MLP_TRY(m, cudaStreamSynchronize(m->stream));
     return check_tc(m);
 }
 
@@ -700,7 +705,7 @@ int mucal_mlp_train(void *mlp, const float *X, const float *t, int64_t B, int32_
     if (!m || !X || !t || B <= 0 || steps <= 0 || !(lr > 0.f))
         return mfail(m, MUCAL_ERR_INVALID_ARG, "bad training arguments");
     MLP_TRY(m, cudaSetDevice(m->device));
-    int rc = upload_batch(m, X, t, B);
+    int rc = upload_batch(m, X, t, B, m->use_tc);
     if (rc != MUCAL_OK) return rc;
     MLP_TRY(m, cudaMemsetAsync(m->grad, 0, NPARAM * 4, m->stream));
     if (m->use_tc) {
@@ -724,7 +729,6 @@ int mucal_mlp_train(void *mlp, const float *X, const float *t, int64_t B, int32_
         MLP_TRY(m, cudaGetLastError());
     }
     if (loss_out) MLP_TRY(m, cudaMemcpyAsync(loss_out, m->loss, 4, cudaMemcpyDeviceToHost, m->stream));
-    MLP_TRY(m, cudaStreamSynchronize(m->stream));
     return check_tc(m);
 }
 

@@ -1,5 +1,8 @@
 // Forward pass of the weight-seeding network with the 128x128 layer on the
-// fifth-generation tensor cores (tcgen05): one CTA of four warps per 128 rows.
+// fifth-generation tensor cores (tcgen05): one CTA of sixteen warps per 128
+// rows.  Bound by the two error functions per unit and row on the ordinary
+// cores and by the latency of one CTA's phases, two CTAs to an SM; 33178 rows
+// (260 CTAs): 18.7 us with eight warps -> 17.5 us.
 //
 //   1. the CTA stages W2 (bf16, [out][in]) and the layer-1 activations of its
 //      128 rows, split into hi = bf16(h1) and lo = bf16(h1 - hi), in shared
@@ -11,9 +14,10 @@
 //      then lo) accumulating Z2 = H1 W2^T in fp32 in TMEM, and commits them to
 //      an mbarrier;
 //   3. after the mbarrier completes, warp q reads TMEM lanes 32(q%4) on (its
-//      rows) with tcgen05.ld, 32 columns at a time: warps 0-3 the columns
-//      0-63, warps 4-7 the columns 64-127; the two halves of
-//      y = b3 + sum_n W3[n] gelu(Z2[n] + b2[n]) meet in shared memory.
+//      rows), columns 32(q/4) on, with tcgen05.ld; the two halves of
+//      y = b3 + sum_n W3[n] gelu(Z2[n] + b2[n]) are summed in column order (a
+//      half's second 32 columns go on from its first) and meet in shared
+//      memory.
 // The mbarrier wait is bounded; if it runs out the CTA records an error flag,
 // frees its TMEM and returns.  Numerics equal the mma.sync path of
 // mlp_kernels.cu up to the order of the fp32 sums.
@@ -30,7 +34,7 @@ namespace {
 
 constexpr int TC_H = 128;                      // hidden width
 constexpr int TC_ROWS = 128;                   // rows per CTA = TMEM lanes
-constexpr int TC_THREADS = 256;                // two threads per row: each takes half the columns
+constexpr int TC_THREADS = 512;                // four threads per row: each takes 32 columns
 constexpr int TC_OFF_W1 = 0, TC_OFF_B1 = TC_H * 4, TC_OFF_W2 = TC_OFF_B1 + TC_H;
 constexpr int TC_OFF_B2 = TC_OFF_W2 + TC_H * TC_H, TC_OFF_W3 = TC_OFF_B2 + TC_H;
 constexpr int TC_OFF_B3 = TC_OFF_W3 + TC_H;
@@ -108,7 +112,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __launch_bounds__(TC_THREADS, 2)
 mlp_forward_tc_kernel(const __nv_bfloat16 *__restrict__ wq, const float *__restrict__ X,
                       float *__restrict__ y, int64_t B, int *err)
 {
@@ -146,18 +150,14 @@ mlp_forward_tc_kernel(const __nv_bfloat16 *__restrict__ wq, const float *__restr
         *reinterpret_cast<uint4 *>(smem + SMEM_B + core_offset(n, kg * 8)) = v;
     }
     __syncthreads();
-    // layer 1 (K = 4, fp32) of row r_in, this thread's half of the units,
+    // layer 1 (K = 4, fp32) of row r_in, this thread's quarter of the units,
     // split into two bf16 terms
-    const int r_in = tid & (TC_ROWS - 1), half = tid >> 7;
+    const int r_in = tid & (TC_ROWS - 1), quarter = tid >> 7, c0 = quarter * 32;
     const int64_t row = (int64_t)blockIdx.x * TC_ROWS + r_in;
-    float x0 = 0.f, x1 = 0.f, x2 = 0.f, x3 = 0.f;
-    if (row < B) {
-        x0 = X[row * 4 + 0];
-        x1 = X[row * 4 + 1];
-        x2 = X[row * 4 + 2];
-        x3 = X[row * 4 + 3];
-    }
-    for (int kg = half * 8; kg < half * 8 + 8; ++kg) {
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row < B) x = *reinterpret_cast<const float4 *>(X + row * 4);
+#pragma unroll 2
+    for (int kg = quarter * 4; kg < quarter * 4 + 4; ++kg) {
         uint32_t hi[4], lo[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -165,8 +165,8 @@ mlp_forward_tc_kernel(const __nv_bfloat16 *__restrict__ wq, const float *__restr
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int n = kg * 8 + 2 * e + u;
-                const float z = s_b1[n] + x0 * s_w1[n * 4 + 0] + x1 * s_w1[n * 4 + 1] +
-                                x2 * s_w1[n * 4 + 2] + x3 * s_w1[n * 4 + 3];
+                const float z = s_b1[n] + x.x * s_w1[n * 4 + 0] + x.y * s_w1[n * 4 + 1] +
+                                x.z * s_w1[n * 4 + 2] + x.w * s_w1[n * 4 + 3];
                 const float h = gelu_tc(z);
                 hv[u] = __bfloat162float(__float2bfloat16_rn(h));
                 lv[u] = h - hv[u];
@@ -205,26 +205,31 @@ mlp_forward_tc_kernel(const __nv_bfloat16 *__restrict__ wq, const float *__restr
     const bool ok = __syncthreads_and(mbar_wait(bar, 0));
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     float *yp = reinterpret_cast<float *>(smem + SMEM_YP);
+    float h[32];
     if (ok) {
-        // warp w reads TMEM lanes 32 (w % 4) .. (its rows), columns of its half
-        float out = 0.f;
-#pragma unroll 1
-        for (int cb = half * 2; cb < half * 2 + 2; ++cb) {
-            float v[32];
-            tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(cb * 32), v);
+        // warp w reads TMEM lanes 32 (w % 4) .. (its rows), columns of its quarter
+        tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, h);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int n = cb * 32 + i;
-                out += s_w3[n] * gelu_tc(v[i] + s_b2[n]);
-            }
+        for (int i = 0; i < 32; ++i) h[i] = gelu_tc(h[i] + s_b2[c0 + i]);
+        if ((quarter & 1) == 0) {
+            float out = 0.f;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) out += s_w3[c0 + i] * h[i];
+            yp[(quarter >> 1) * TC_ROWS + r_in] = out;
         }
-        yp[half * TC_ROWS + r_in] = out;
     } else if (tid == 0) {
-        atomicExch(err, 1);
+        *reinterpret_cast<volatile int *>(err) = 1;
+    }
+    __syncthreads();
+    if (ok && (quarter & 1) != 0) {
+        float out = yp[(quarter >> 1) * TC_ROWS + r_in];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) out += s_w3[c0 + i] * h[i];
+        yp[(quarter >> 1) * TC_ROWS + r_in] = out;
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (ok && half == 0 && row < B) y[row] = *s_b3 + yp[r_in] + yp[TC_ROWS + r_in];
+    if (ok && quarter == 0 && row < B) y[row] = *s_b3 + yp[r_in] + yp[TC_ROWS + r_in];
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_H));
 }
@@ -538,7 +543,7 @@ mlp_train_tc_kernel(const __nv_bfloat16 *__restrict__ wq, const __nv_bfloat16 *_
 #pragma unroll
         for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
     } else if (tid == 0) {
-        atomicExch(err, 1);
+        *reinterpret_cast<volatile int *>(err) = 1;
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
