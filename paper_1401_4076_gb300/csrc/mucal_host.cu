@@ -548,6 +548,7 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
         const int rc = ensure_thr_transposed(c);
         if (rc != MUCAL_OK) return rc;
     }
+    CUDA_TRY(c, mucal::walker_update_allow_smem(sh, c->max_smem));
     int rc = build_work(c, sh);
     if (rc != MUCAL_OK) return rc;
     c->shape = sh;

@@ -73,12 +73,10 @@ struct ReduceWork {
     int32_t row0;
 };
 
-// Walker-update kernels of one (tunnelling, persistent) flavour: the thread
-// kernel in its shared-memory variants, the group kernel with the bitsets in
-// shared or global memory and the thresholds in global memory, in shared
-// memory or in a per-walker row window, and the field kernel with the three
-// threshold modes.
-constexpr int kWalkerUpdateFns = 4 + 5 * 2 * 3 + 5 * 3;
+// Static shared memory of the walker-update kernels (the largest: a word per
+// thread of a block and the persistent launches' work item, on 16 bytes).
+constexpr int kWalkerStaticSmem = 2064;
+
 // Kernels of one lane count with several commits per round (persistent or
 // not, tunnelling bookkeeping or not): bitsets in shared memory, in global
 // memory or count fields, each with the thresholds in global memory, in
@@ -118,15 +116,10 @@ cudaError_t launch_walker_update(const SysParams *dev_sys, const BlockWork *dev_
                                  bool tunnel, int grid, int *next_item, cudaStream_t stream);
 // The other three flavours of the walker update, one translation unit each
 // (walker_kernels_tun.cu, walker_kernels_persist.cu,
-// walker_kernels_persist_tun.cu): the kernel of a launch shape and all
-// kWalkerUpdateFns kernels of the flavour (for their shared-memory
-// attributes).
+// walker_kernels_persist_tun.cu).
 const void *walker_update_fn_tunnel(const LaunchShape &shape);
-void walker_update_tunnel_fns(const void *(&fns)[kWalkerUpdateFns]);
 const void *walker_update_fn_persist(const LaunchShape &shape);
-void walker_update_persist_fns(const void *(&fns)[kWalkerUpdateFns]);
 const void *walker_update_fn_persist_tun(const LaunchShape &shape);
-void walker_update_persist_tun_fns(const void *(&fns)[kWalkerUpdateFns]);
 // The kernels with several commits per round, one translation unit per lane
 // count (walker_scan_<lanes>.cu), in the order of kWalkerScanFns.
 void walker_scan_4_fns(const void *(&fns)[kWalkerScanFns]);
@@ -143,7 +136,11 @@ size_t thr_window_bytes(const SysParams &p);
 size_t field_smem_bytes(const SysParams &p);
 cudaError_t launch_hist_reduce(const SysParams *dev_sys, const ReduceWork *dev_work, int n_items,
                                cudaStream_t stream);
+// Dynamic shared memory a walker-update block can have, and the leave to use
+// that much for the kernels of one shape (asking for every kernel at every
+// context creation took 0.3 ms).
 cudaError_t walker_update_max_smem(int *bytes);
+cudaError_t walker_update_allow_smem(const LaunchShape &shape, int bytes);
 // Rewrite the dE-major copy of system p's threshold table from p.thr.
 cudaError_t launch_thr_transpose(const SysParams &p, cudaStream_t stream);
 

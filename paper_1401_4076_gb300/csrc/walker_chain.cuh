@@ -1,8 +1,9 @@
 // Device code of the walker update shared by the translation units that
 // instantiate it: walker_kernels.cu (plain), walker_kernels_tun.cu (with
 // tunnelling bookkeeping), walker_kernels_persist.cu and
-// walker_kernels_persist_tun.cu (persistent launches).  Everything here has internal linkage; each unit
-// gets its own copy of what it instantiates.
+// walker_kernels_persist_tun.cu (persistent launches), and walker_scan.cuh
+// with its rounds of several commits.  Everything here has internal linkage;
+// each unit gets its own copy of what it instantiates.
 //
 // The threshold rows a walker's acceptance test reads come from the table in
 // global memory, from the whole table staged in shared memory, or (group and
@@ -1196,8 +1197,7 @@ const void *group_fn(const LaunchShape &sh)
     return sh.bits_in_smem ? group_fn_sb<G, true, TUN, PE>(sh) : group_fn_sb<G, false, TUN, PE>(sh);
 }
 
-// The kernel of a launch shape among the kWalkerUpdateFns of one (TUN, PE) flavour
-// (PE: persistent launch); the caller checks that shape.persistent == PE.
+// The kernel of a launch shape in one (TUN, PE) flavour (PE: persistent launch); the caller checks that shape.persistent == PE.
 template <bool TUN, bool PE>
 const void *walker_update_fn_t(const LaunchShape &sh)
 {
@@ -1225,41 +1225,6 @@ const void *walker_update_fn_t(const LaunchShape &sh)
     case 32: return group_fn<32, TUN, PE>(sh);
     default: return nullptr;
     }
-}
-
-// Every walker-update kernel of one (TUN, PE) flavour (for their
-// shared-memory attributes).
-template <bool TUN, bool PE>
-void walker_update_fns(const void *(&fns)[kWalkerUpdateFns])
-{
-    int i = 0;
-    fns[i++] = (const void *)walker_update_thread<true, true, TUN, PE>;
-    fns[i++] = (const void *)walker_update_thread<true, false, TUN, PE>;
-    fns[i++] = (const void *)walker_update_thread<false, true, TUN, PE>;
-    fns[i++] = (const void *)walker_update_thread<false, false, TUN, PE>;
-#define MUCAL_GROUP_FNS(G)                                                          \
-    fns[i++] = (const void *)walker_update_group<G, true, kThrShared, TUN, PE>;    \
-    fns[i++] = (const void *)walker_update_group<G, true, kThrGlobal, TUN, PE>;    \
-    fns[i++] = (const void *)walker_update_group<G, true, kThrWindow, TUN, PE>;    \
-    fns[i++] = (const void *)walker_update_group<G, false, kThrShared, TUN, PE>;   \
-    fns[i++] = (const void *)walker_update_group<G, false, kThrGlobal, TUN, PE>;   \
-    fns[i++] = (const void *)walker_update_group<G, false, kThrWindow, TUN, PE>;
-    MUCAL_GROUP_FNS(2)
-    MUCAL_GROUP_FNS(4)
-    MUCAL_GROUP_FNS(8)
-    MUCAL_GROUP_FNS(16)
-    MUCAL_GROUP_FNS(32)
-#undef MUCAL_GROUP_FNS
-#define MUCAL_FIELD_FNS(G)                                                     \
-    fns[i++] = (const void *)walker_update_field<G, kThrShared, TUN, PE>;     \
-    fns[i++] = (const void *)walker_update_field<G, kThrGlobal, TUN, PE>;     \
-    fns[i++] = (const void *)walker_update_field<G, kThrWindow, TUN, PE>;
-    MUCAL_FIELD_FNS(2)
-    MUCAL_FIELD_FNS(4)
-    MUCAL_FIELD_FNS(8)
-    MUCAL_FIELD_FNS(16)
-    MUCAL_FIELD_FNS(32)
-#undef MUCAL_FIELD_FNS
 }
 
 }  // namespace

@@ -338,37 +338,17 @@ cudaError_t walker_update_max_smem(int *bytes)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
-    const void *fl[4][kWalkerUpdateFns];
-    walker_update_fns<false, false>(fl[0]);
-    walker_update_tunnel_fns(fl[1]);
-    walker_update_persist_fns(fl[2]);
-    walker_update_persist_tun_fns(fl[3]);
-    const void *sc[4][kWalkerScanFns];
-    walker_scan_4_fns(sc[0]);
-    walker_scan_8_fns(sc[1]);
-    walker_scan_16_fns(sc[2]);
-    walker_scan_32_fns(sc[3]);
-    const void *fns[4 * (kWalkerUpdateFns + kWalkerScanFns)];
-    int n = 0;
-    for (int f = 0; f < 4; ++f) {
-        for (const void *fn : fl[f]) fns[n++] = fn;
-        for (const void *fn : sc[f]) fns[n++] = fn;
-    }
-    // the dynamic limit leaves room for the largest static shared array (the
-    // thread kernel's tunnelling words)
-    size_t max_static = 0;
-    for (const void *fn : fns) {
-        cudaFuncAttributes attr{};
-        e = cudaFuncGetAttributes(&attr, fn);
-        if (e != cudaSuccess) return e;
-        max_static = attr.sharedSizeBytes > max_static ? attr.sharedSizeBytes : max_static;
-    }
-    *bytes -= (int)max_static;
-    for (const void *fn : fns) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, *bytes);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    *bytes -= kWalkerStaticSmem;
+    return e;
+}
+
+cudaError_t walker_update_allow_smem(const LaunchShape &shape, int bytes)
+{
+    for (int tunnel = 0; tunnel < 2; ++tunnel) {
+        const void *fn = walker_update_fn(shape, tunnel != 0);
+        if (!fn) return cudaErrorInvalidValue;
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
