@@ -114,6 +114,10 @@ typedef struct mucal_system_desc {
     uint64_t seed_base; /* walker w uses Philox key seed_base + w */
 } mucal_system_desc;
 
+/* A new context has a shape chosen from its systems' sizes and walkers: several
+   commits per round (from 16 particles up), as many walkers side by side as
+   there are or as shared memory holds.  The defaults below are those of a
+   configuration that names only some fields. */
 typedef struct mucal_launch_config {
     int32_t kernel;            /* MUCAL_KERNEL_THREAD, _GROUP or _FIELD */
     int32_t lanes_per_walker;  /* 1 for THREAD; 2, 4, 8, 16 or 32 for GROUP and FIELD */
@@ -138,16 +142,18 @@ typedef struct mucal_launch_config {
                                   (mucal_get_launch_config then reports 0, as it does
                                   when the whole table is staged in shared memory).
                                   Ignored by THREAD.  Default 1 */
-    int32_t multi_commit;      /* GROUP and FIELD kernels with 4 or more lanes and the
-                                  thresholds in global or shared memory (no row
-                                  windows): 1 = one round of G proposals may commit
-                                  several accepted moves in order, each lane re-deciding
-                                  against the energy its predecessors left while its
-                                  move stays independent of theirs; 0 = one commit per
-                                  round.  Both give the same chain (Sec. 2's Metropolis
-                                  sequence, bit-identical).  With tunnelling events
-                                  recorded the one-commit rounds run.  Reported as 0
-                                  where it does not apply.  Default 0 */
+    int32_t multi_commit;      /* GROUP and FIELD kernels with 4 or more lanes and
+                                  thr_window 0, or a table that is staged whole: 1 = the
+                                  lanes hold a sliding window of as many attempts, and a
+                                  round decides and commits all up to the first one that
+                                  an earlier accepted move touches; where the table is
+                                  not staged, each walker keeps the rows around its
+                                  energy in shared memory if they fit beside the block's
+                                  walkers, else the thresholds are read from global
+                                  memory; 0 = one commit per round.  Both give the same
+                                  chain (Sec. 2's Metropolis sequence, bit-identical),
+                                  with and without tunnelling events.  Reported as 0
+                                  where it does not apply.  0 unless given */
 } mucal_launch_config;
 
 typedef struct mucal_system_info {

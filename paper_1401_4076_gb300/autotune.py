@@ -107,7 +107,7 @@ def with_threshold_modes(cands):
     """Every group and field candidate also with thr_window = 0 (thresholds
     read from global memory when the table does not fit in shared memory;
     the default 1 keeps a window of rows per walker there instead), and at
-    4 lanes or more with multi-commit rounds (which read the rows directly)."""
+    4 lanes or more with multi-commit rounds (which keep rows of their own)."""
     out = []
     for c in cands:
         out.append(c)

@@ -565,13 +565,19 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
 // L = 33, N = 3244, r = 1: 8.86 / 5.06 / 3.37 / 2.85; 3D L = 24, N = 1382,
 // r = 14: 7.75 / 4.51 / 3.82 / 6.9; 3D L = 32, N = 3277, r = 28: 18.3 / 12.4 /
 // 13.0 / -; 2D L = 64, N = 410, r = 1: 4.29 / 2.74 / 2.28 / 2.79, r = 10: 4.35 /
-// 2.80 / 3.05 / 7.3; 3D L = 8, N = 56, r = 56: 1.44 / 1.98 / 5.2 / -; 2D
-// L = 14, N = 17, r = 19: 0.51 / 0.65 / 1.40 / -.
+// 2.80 / 3.05 / 7.3; 3D L = 8, N = 56, r = 56: 1.44 / 1.98 / 5.2 / -.
+// Narrow windows pay while moves are accepted; where they are refused, wide
+// ones pass over more at a time.  At acceptance 0.8 and 0.04 (with one commit
+// per round, 8 lanes, behind it): 2D L = 14, N = 24, r = 20: 4 lanes 0.51 and
+// 0.31, 8 lanes 0.71 and 0.22 (0.68, 0.22); 2D L = 20, N = 20, r = 7: 0.39 and
+// 0.27, 0.37 and 0.18 (0.46, 0.17); 2D L = 40, N = 100, r = 60: 0.83 and 0.46,
+// 0.79 and 0.38 (1.03, 0.39); 2D L = 40, N = 60, r = 1, 16 lanes: 0.55 and 0.19
+// (0.81, 0.26).
 int default_lanes(long long r, double N)
 {
-    if (N < 32 || (N < 200 && r > 48)) return 4;
+    if ((N < 48 && r >= 12) || (N < 64 && r > 48)) return 4;
     if (N >= 2500 && r <= 7) return 32;
-    if ((N >= 1000 && r <= 24) || (N >= 300 && r <= 4)) return 16;
+    if ((N >= 1000 && r <= 24) || (N >= 60 && r <= 4)) return 16;
     return 8;
 }
 

@@ -28,16 +28,28 @@ namespace {
 // attempt is never stopped, so every round decides at least one, mostly the
 // whole window; no group of a warp waits for another's conflicts.
 //
+// Where the last round had few accepted moves in each walker of the warp, a
+// round takes all decisions at its first energy, one threshold a lane, and
+// ends with the first accepted attempt: no recurrence, no tests for touching,
+// one commit to look for in the lists.  (Rounds of the recurrence without the
+// tests for touching took, at 2D L = 40, N = 60, 64 walkers, 60 sweeps and
+// acceptance 0.03, 0.254 ms, these 0.149; 2D L = 16, N = 32 at 0.04 0.319 and
+// 0.209, rounds that always end at the first accepted attempt 0.223.  Few is a
+// quarter of the window: an eighth 0.155 and 0.227, more than a quarter of the
+// warp's attempts together instead 2D L = 64 1.12 -> 1.43 at 0.45.)
+//
 // The rounds are bound by the latency of dependent integer instructions and by
 // issue slots (a walker is one serial chain, and an SM holds only tens of
-// walkers): on 2D L = 64 at 8 lanes and 28 walkers per SM a round is about 540
+// walkers): on 2D L = 64 at 8 lanes and 28 walkers per SM a round was about 540
 // warp instructions, one issued every 4.0 cycles per warp, for 7.3 attempts
 // per walker (18.3 warp instructions per attempt against 24 with one commit
-// per round; 2.9e10 against 1.7e10 attempts/s).  So independent work stands
-// beside the recurrence, in the same straight line of code: the random
-// numbers (2.77e10 -> 2.86e10 attempts/s) and the comparisons of the moves'
-// sites (-> 2.95e10).  Two attempts per lane, which halve what is done once
-// per lane, issued as much and ran at half the warps: 2.07e10.
+// per round).  So independent work stands beside the recurrence, in the same
+// straight line of code: the random numbers (2.77e10 -> 2.86e10 attempts/s)
+// and the comparisons of the moves' sites (-> 2.95e10; one commit per round
+// 1.7e10); with the rounds of few moves a path of their own the others have
+// fewer instructions to choose between (20 sweeps 1.22 -> 1.15 ms).  Two attempts
+// per lane, which halve what is done once per lane, issued as much and ran at
+// half the warps: 2.07e10.
 //
 // A step of the recurrence is one threshold load from shared memory and a few
 // dependent integer instructions: from the whole table (kThrShared), or from
@@ -50,9 +62,12 @@ namespace {
 // attempt is stopped when reached with another energy.
 // ---------------------------------------------------------------------------
 constexpr int kScanWords = 24;    // energies of a decision mask (bits 0-23; the lane's dE above)
-constexpr int kScanFew = 2;       // accepted moves of a walker's round that are still few
-constexpr int kScanDrift = 5;     // a window's centre follows an energy further from it than this
 constexpr int kScanReach = 10;    // of which at least this many on either side of the round's energy
+template <int W>
+constexpr int kScanFew = W / 4;   // accepted moves of a walker's round that are still few
+// A window's centre follows an energy further from it than this (ms of 3D
+// L = 32, N = 3277, 8192 walkers, 10 sweeps at 5 / 7 / 9 rows: 12.81 / 12.40 / 12.23).
+constexpr int kScanDrift = 9;
 static_assert(kThrTPad >= kScanReach + 3 && kThrTPad >= kScanWords - kScanReach, "window in the padding");
 
 // Occupation as the rounds read it: de() is the energy change but for the
@@ -383,25 +398,8 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
         mn = decided ? mq : mn;
         r2n = decided ? r2q : r2n;
     };
-    bool many = true;            // (the same in the whole warp) how the last round went:
-    bool quiet = false;          // many accepted moves, or none in the whole warp
+    bool many = true;            // (the same in the whole warp) the last round had many accepted moves
     while (__any_sync(FULL, active && t0 < A)) {
-        // As long as no walker of the warp moves there is nothing to try for
-        // conflicts, commit or patch: rounds of the recurrence alone (a round
-        // that meets an accepted move is begun again below).
-        while (quiet) {
-            begin();
-            recurrence();
-            prefetch();
-            if (__any_sync(FULL, (am & places()) != 0u)) break;
-            const uint32_t nd = near < W ? near : (uint32_t)W;
-            advance(place < nd);
-            carry += nd;
-            t0 += nd;
-            const bool more = __any_sync(FULL, active && t0 < A);
-            const bool full = __any_sync(FULL, carry >= 0x40000000u);   // (recorded below)
-            quiet = more && !full;
-        }
         if constexpr (TM == kThrWindow) {
             // rows asked for a round ago; then the window follows the energy
             if (active && t0 < A) {
@@ -427,11 +425,72 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
             }
         }
         begin();
-        // After a round with many accepted moves, every pair of slots is tried
-        // ahead of the recurrence, slot s against the W / 2 behind it in the
-        // ring; after one with few, only the accepted ones are tried, after it.
+        const unsigned bit = 1u << place;
+        const uint32_t nv = near < W ? near : (uint32_t)W;
+        if (!many) {
+            // Few accepted moves: the decisions at the round's energy alone,
+            // one threshold a lane, up to the first accepted attempt.
+            uint32_t T;
+            if constexpr (TM == kThrGlobal) {
+                T = __ldg(thr + ((place < near ? code : 0u) * pitch + (uint32_t)(bin + kThrTPad)));
+            } else {
+                const uint32_t row = TM == kThrWindow ? (uint32_t)bin & (kThrWindowRows - 1u) : (uint32_t)bin;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(T) : "r"(row * (4u * TS) + (rbase + 4u * code)));
+            }
+            draw(t0 + place + 2 * W, kq, mq, r2q);
+            prefetch();
+            const unsigned votes = __ballot_sync(FULL, place < nv && T >= r2p);
+            if (votes == 0u) {
+                advance(place < nv);
+                carry += nv;
+                t0 += nv;
+            } else {
+                const unsigned mine = (votes >> gbase) & GMASK;
+                am = turn_left<W>(mine, (uint32_t)W - h);
+                many = __any_sync(FULL, __popc(am) > kScanFew<W>);
+                const uint32_t first = am ? (uint32_t)__ffs(am) - 1u : 0u;
+                const uint32_t nd = am ? first + 1u : nv;
+                const int src = gbase + (int)((first + h) & WM);
+                const uint32_t cc = __shfl_sync(FULL, code, src);
+                uint32_t ck, cm, ca, cb;
+                shfl_pair<IdxT>(k, m, src, ck, cm);
+                shfl_pair<IdxT>(a, b, src, ca, cb);
+                const int de = am ? (int)cc - 2 * D : 0;
+                if (am && place == first) {
+                    v.commit(a, b, na, nb);
+                    S[k] = (IdxT)b;
+                    S[N + m] = (IdxT)a;
+                    ++acc;
+                    const uint32_t cnt = carry + first;
+                    if (de != 0 && cnt != 0u) atomicAdd(hist + bin, (unsigned long long)cnt);
+                }
+                carry = de != 0 ? 1u : carry + nd;
+                bin += de;
+                if (tun && am) {
+                    if (bin <= tlo) {
+                        tcnt += tst == 2u ? 1u : 0u;
+                        tst = 1u;
+                    } else if (bin >= thi) {
+                        tcnt += tst == 1u ? 1u : 0u;
+                        tst = 2u;
+                    }
+                }
+                advance(place < nd);
+                a = am && ck == k ? cb : a;
+                b = am && cm == m ? ca : b;
+                t0 += nd;
+            }
+            if (carry >= 0x40000000u) {
+                if (active && j == 0) atomicAdd(hist + bin, (unsigned long long)carry);
+                carry = 0;
+            }
+            __syncwarp(FULL);
+            continue;
+        }
+        // Many: every pair of slots is tried for touching ahead of the
+        // recurrence, slot s against the W / 2 behind it in the ring.
         unsigned behind = 0;       // places of the touched ones
-        if (many) {
+        {
             uint32_t pa[W / 2], pb[W / 2];
             __syncwarp(FULL);
             stage[j] = PAIR ? (a | (b << 16)) : a;
@@ -455,8 +514,6 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
             for (int d = 1; d <= W / 2; ++d)
                 or_if_touch<D>(c, 1u << (d - 1), na, nb, a, b, pa[d - 1], pb[d - 1]);
             behind = turn_left<W>(c, place + 1);
-        } else {
-            recurrence();
         }
         prefetch();
         // the energy bin after the own attempt
@@ -470,7 +527,6 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
         const int x1 = (int)stage[place];
         // attempts that have to wait (bad) and those whose move changes the
         // energy (up), by place, over the group
-        const unsigned bit = 1u << place;
         const int de = (int)code - 2 * D;
         const bool yes = (am & bit) != 0u && place < near;
         const int x = x1 - (yes ? de : 0);
@@ -478,20 +534,8 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
         if constexpr (TM == kThrGlobal) bad |= (uint32_t)(x - bin + x0) >= (uint32_t)kScanWords ? bit : 0u;
         if constexpr (TM == kThrWindow) bad |= x < vlo || x > vhi ? bit : 0u;
         am &= places();
-        if (many) {
-            bad |= (behind & am & (bit - 1u)) ? bit : 0u;
-            bad |= yes ? behind & ~(bit | (bit - 1u)) : 0u;
-        } else {
-            unsigned todo = am;
-            while (__any_sync(FULL, todo != 0u)) {
-                const uint32_t i = todo ? (uint32_t)__ffs(todo) - 1u : 0u;
-                const uint32_t slot = (i + h) & WM;
-                uint32_t pa, pb;
-                shfl_pair<IdxT>(a, b, gbase + (int)slot, pa, pb);
-                or_if_touch<D>(bad, todo != 0u && place > i ? bit : 0u, na, nb, a, b, pa, pb);
-                todo &= todo - 1u;
-            }
-        }
+        bad |= (behind & am & (bit - 1u)) ? bit : 0u;
+        bad |= yes ? behind & ~(bit | (bit - 1u)) : 0u;
         if constexpr (W <= 16) {
             unsigned y = bad | (up << 16);
 #pragma unroll
@@ -506,13 +550,10 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
             }
         }
         // attempts decided (a bad one past the end is none)
-        const uint32_t nv = near < W ? near : (uint32_t)W;
         const uint32_t nd = bad ? min((uint32_t)__ffs(bad) - 1u, nv) : nv;
         const unsigned done = W == 32 && nd >= 32u ? 0xffffffffu : (1u << nd) - 1u;
         const unsigned chg = up & done;
-        many = __any_sync(FULL, __popc(am) > kScanFew);
-        quiet = false;
-        if (!many) quiet = !__any_sync(FULL, am != 0u);
+        many = __any_sync(FULL, __popc(am) > kScanFew<W>);
         const bool commit = yes && place < nd;
         // the list slots a commit rewrites
         const uint32_t moved = commit && PAIR ? (k | (m << 16)) : 0xFFFFFFFFu;   // (indices below 65535)

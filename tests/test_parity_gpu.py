@@ -747,3 +747,63 @@ def test_histogram_rows_grow_with_the_launch_shape():
             mc.run_iteration(3, it)
             hist, _ = chain.run_walkers(2, 16, 32, 0, it, 96, -64, 0, T, S, occ, E)
             np.testing.assert_array_equal(mc.histogram(0), hist.sum(axis=0))
+
+
+# ----------------------------------------------- rounds with several commits
+
+@pytest.mark.parametrize("desc,sweeps,launch", [
+    # whole table staged: every window width, 21 and 111 attempts
+    ((2, 8, 3, 9, 0, 0, 3), 7, dict(kernel=m.MUCAL_KERNEL_GROUP, lanes_per_walker=4, walkers_per_block=8)),
+    ((2, 12, 37, 9, 0, 0, 4), 3, dict(kernel=m.MUCAL_KERNEL_FIELD, lanes_per_walker=8, walkers_per_block=4)),
+    ((3, 7, 37, 5, 0, 0, 5), 3, dict(kernel=m.MUCAL_KERNEL_GROUP, lanes_per_walker=16, walkers_per_block=2)),
+    ((2, 12, 37, 5, 0, 0, 6), 3, dict(kernel=m.MUCAL_KERNEL_FIELD, lanes_per_walker=32, walkers_per_block=1)),
+    # rows of their own: tables of 5003 and 3604 rows
+    ((2, 90, 2501, 5, 0, 0, 7), 1, dict(kernel=m.MUCAL_KERNEL_GROUP, lanes_per_walker=8, walkers_per_block=4)),
+    ((3, 17, 1201, 5, 0, 0, 8), 1, dict(kernel=m.MUCAL_KERNEL_FIELD, lanes_per_walker=16, walkers_per_block=2)),
+    # nor those beside eight fields of 27000 bytes: masks from global memory
+    ((3, 30, 1201, 11, 0, 0, 9), 1, dict(kernel=m.MUCAL_KERNEL_FIELD, lanes_per_walker=8, walkers_per_block=8)),
+    # 32-bit lists
+    ((2, 257, 301, 3, 0, 0, 10), 3, dict(kernel=m.MUCAL_KERNEL_GROUP, lanes_per_walker=4, walkers_per_block=8)),
+], ids=lambda x: f"L{x[1]}" if isinstance(x, tuple) else None)
+def test_scan_rounds_bit_exact(desc, sweeps, launch):
+    """Iterations in which most moves are taken, few, none, and most again,
+    with tunnelling events: the rounds with many accepted moves, those up to
+    the first one, and the changes between them."""
+    d, L, N, W, lo, hi, seed = desc
+    e_min = -N // 8
+    S, occ, E = _oracle_states(d, L, N, W, seed)
+    tstate, tcount = np.zeros(W, np.uint8), np.zeros(W, np.int64)
+    grid = np.arange(-d * N, 1, dtype=np.float64)
+    with m.Mucal([desc], per_walker_hist=True) as mc:
+        mc.set_launch(bits_in_smem=1, thr_window=0, multi_commit=1, **launch)
+        assert mc.launch()["multi_commit"] == 1
+        mc.set_tunnel_window(0, e_min, 0)
+        for it, beta in enumerate((0.0, 2.0, 3.5, 40.0, 0.3)):
+            lnW = -beta * grid
+            mc.set_weights(0, lnW)
+            T = chain.thresholds(d, -d * N, 0, lnW)
+            mc.run_iteration(sweeps, it)
+            hist = chain.run_walkers_tunnel(d, L, N, seed, it, sweeps * N, -d * N, 0, T, S, occ, E,
+                                            e_min, 0, tstate, tcount)
+            _, per = mc.histogram(0, per_walker=True)
+            np.testing.assert_array_equal(per, hist)
+        np.testing.assert_array_equal(mc.tunnel_counts(0)[1].astype(np.int64), tcount)
+        for w in range(W):
+            _assert_walker_equal(mc, 0, w, S[w], occ[w], E[w])
+
+
+@pytest.mark.parametrize("desc", [(2, 14, 15, 64, 0, 0, 1), (2, 1000, 1000, 4, 0, 0, 2),
+                                  (3, 64, 2000, 3, 0, 0, 3)])
+def test_default_shape_bit_exact(desc):
+    """The shape of a new context at the ends of its rule: one commit per round
+    below 16 particles, bitsets that fill a block, and lists of 32 bits."""
+    d, L, N, W, lo, hi, seed = desc
+    S, occ, E = _oracle_states(d, L, N, W, seed)
+    T = chain.thresholds(d, -d * N, 0, np.zeros(d * N + 1))
+    with m.Mucal([desc]) as mc:
+        assert mc.launch()["multi_commit"] == (0 if N < 16 else 1)
+        mc.run_iteration(1, 0)
+        hist, _ = chain.run_walkers(d, L, N, seed, 0, N, -d * N, 0, T, S, occ, E)
+        np.testing.assert_array_equal(mc.histogram(0), hist.sum(axis=0))
+        for w in range(W):
+            _assert_walker_equal(mc, 0, w, S[w], occ[w], E[w])
