@@ -599,9 +599,11 @@ int default_lanes(long long r, double N)
 // resident walker: 2D L = 64 3.24 (bitsets) -> 3.11, but five 2D systems of
 // L = 61 to 97, 5120 walkers, 50 sweeps 1.06 (bitsets) against 1.9.
 //
-// Below 16 particles nearly every window holds a conflict, and the rounds with
-// one commit are as fast or faster: 2D L = 22, N = 12, 64 walkers 0.122 against
-// 0.122 ms at acceptance 0.5, 0.089 against 0.116 at 0.1.
+// Below 12 particles nearly every window holds a conflict, and the rounds with
+// one commit are faster (8 lanes, ms at a high and a middle acceptance, one
+// against several commits): 2D L = 10, N = 8, 64 walkers 0.63 and 0.42 against
+// 0.77 and 0.49; 2D L = 22, N = 12, 64 walkers 0.59 and 0.51 against 0.53 and
+// 0.45, 3000 walkers 0.73 and 0.62 against 0.52 and 0.48 (4 lanes).
 mucal_launch_config default_launch(Context *c)
 {
     long long total = 0;
@@ -659,7 +661,7 @@ mucal_launch_config default_launch(Context *c)
             cap = f;
         }
     }
-    if (N < 16) {
+    if (N < 12) {
         def.multi_commit = 0;
         def.thr_window = 1;
         if (!plain_fits(def.kernel)) def.bits_in_smem = 0;

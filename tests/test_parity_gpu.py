@@ -792,16 +792,16 @@ def test_scan_rounds_bit_exact(desc, sweeps, launch):
             _assert_walker_equal(mc, 0, w, S[w], occ[w], E[w])
 
 
-@pytest.mark.parametrize("desc", [(2, 14, 15, 64, 0, 0, 1), (2, 1000, 1000, 4, 0, 0, 2),
-                                  (3, 64, 2000, 3, 0, 0, 3)])
+@pytest.mark.parametrize("desc", [(2, 14, 11, 64, 0, 0, 1), (2, 14, 12, 64, 0, 0, 4),
+                                  (2, 1000, 1000, 4, 0, 0, 2), (3, 64, 2000, 3, 0, 0, 3)])
 def test_default_shape_bit_exact(desc):
     """The shape of a new context at the ends of its rule: one commit per round
-    below 16 particles, bitsets that fill a block, and lists of 32 bits."""
+    below 12 particles, bitsets that fill a block, and lists of 32 bits."""
     d, L, N, W, lo, hi, seed = desc
     S, occ, E = _oracle_states(d, L, N, W, seed)
     T = chain.thresholds(d, -d * N, 0, np.zeros(d * N + 1))
     with m.Mucal([desc]) as mc:
-        assert mc.launch()["multi_commit"] == (0 if N < 16 else 1)
+        assert mc.launch()["multi_commit"] == (0 if N < 12 else 1)
         mc.run_iteration(1, 0)
         hist, _ = chain.run_walkers(d, L, N, seed, 0, N, -d * N, 0, T, S, occ, E)
         np.testing.assert_array_equal(mc.histogram(0), hist.sum(axis=0))
