@@ -391,7 +391,7 @@ struct ThrWindow {
     // rounds then read stale rows; the host reports the iteration invalid).
     __device__ __forceinline__ void wait(const SysParams &p)
     {
-        if (!pend) return;
+        if (!pend || broken) return;
         uint32_t ok = 0;
         for (uint32_t i = 0; i < kWaitLimit && !ok; ++i) ok = mbar_try_wait(mbar, phase);
         if (!ok) {
@@ -401,6 +401,17 @@ struct ThrWindow {
         }
         phase ^= 1u;
         pend = false;
+    }
+
+    // The same for the lanes gm of a group (all of them call), with one outcome
+    // for all: each lane polls by itself, so a copy that lands at the limit
+    // can run out for some of them only, and lanes that go on from different
+    // attempts would keep each other's rounds from ever deciding one.
+    __device__ __forceinline__ void wait_group(const SysParams &p, unsigned gm)
+    {
+        if (!pend || broken) return;
+        wait(p);
+        broken = __any_sync(gm, broken) != 0;
     }
 };
 

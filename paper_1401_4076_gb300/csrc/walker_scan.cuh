@@ -266,7 +266,7 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
             if (j == 0) mbar_init(mbar_s, 1u);
             __syncwarp(gm);
             tw.fetch(bin - WLO, bin + WHI, j == 0);
-            tw.wait(p);
+            tw.wait_group(p, gm);
         }
         vlo = bin - WLO;
         vhi = bin + WHI;
@@ -404,24 +404,25 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
             // rows asked for a round ago; then the window follows the energy
             if (active && t0 < A) {
                 if (tw.pend) {
-                    tw.wait(p);
+                    tw.wait_group(p, gm);
                     vlo = tw.c - WLO;
                     vhi = tw.c + WHI;
                 }
                 const int off = bin - tw.c;
-                if (off > kScanDrift || off < -kScanDrift) {
+                if (!tw.broken && (off > kScanDrift || off < -kScanDrift)) {
                     if (off > 0) tw.fetch(max(tw.c + WHI + 1, bin - WLO), bin + WHI, j == 0);
                     else tw.fetch(bin - WLO, min(tw.c - WLO - 1, bin + WHI), j == 0);
                     vlo = max(vlo, bin - WLO);
                     vhi = min(vhi, bin + WHI);
                     tw.c = bin;
-                    if (tw.pend && (bin < vlo || bin > vhi)) tw.wait(p);
+                    if (tw.pend && (bin < vlo || bin > vhi)) tw.wait_group(p, gm);
                     if (!tw.pend) {
                         vlo = bin - WLO;
                         vhi = bin + WHI;
                     }
                 }
-                if (tw.broken) t0 = A;     // the walker stops; the host reports the iteration invalid
+                // the walker stops, in all lanes of its group; the host reports the iteration invalid
+                if (tw.broken) t0 = A;
             }
         }
         begin();
@@ -643,11 +644,11 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
     if constexpr (TM == kThrWindow) {
         if (active) {
             // no copy may still write into the ring when the block moves on
-            if (tw.broken) {
+            if (!tw.broken) {
+                tw.wait_group(p, gm);
+            } else if (tw.pend) {
                 uint32_t ok = 0;
                 for (uint32_t i = 0; i < kWaitLimit && !ok; ++i) ok = mbar_try_wait(mbar_s, tw.phase);
-            } else {
-                tw.wait(p);
             }
             __syncwarp(gm);
             if (j == 0) mbar_inval(mbar_s);
