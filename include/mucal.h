@@ -302,7 +302,9 @@ int mucal_get_stats(void *ctx, int32_t sys, mucal_stats *stats);
 
 /* Device pointer of the summed histogram H(E) of system sys (int64[n_bins],
  * library-owned, valid until mucal_destroy; contents valid once the
- * context's stream has finished the last mucal_run_iteration). */
+ * context's stream has finished the last mucal_run_iteration).  What the
+ * caller has written to it, finished before the call, counts in the system's
+ * first read or weight update after an iteration. */
 int mucal_histogram_device_ptr(void *ctx, int32_t sys, void **dptr);
 
 /* Library version string. */

@@ -39,6 +39,8 @@ struct System {
     uint32_t *thr_pinned = nullptr; // staging buffer of the threshold upload
     size_t thr_count = 0;
     size_t h_off = 0;               // its place in the context's summed histograms
+    bool hist_ahead = false;        // H came with another system's read, not asked for yet
+    bool hist_shared = false;       // the caller has the device histogram's address
     uint64_t last_attempts = 0;
     std::vector<double> lnW_run;    // the weights of the last iteration's thresholds
     unsigned long long *drop_acc = nullptr;  // device [3][n_bins] droplet accumulators
@@ -696,10 +698,13 @@ int check_sys(Context *c, int32_t s)
 
 // Every system's summed histogram to the host, with the error flag behind
 // them, by one copy into pinned memory (a copy per system and one for the
-// flag, both pageable, cost an 8-system tempering round 0.13 ms).
+// flag, both pageable, cost an 8-system tempering round 0.13 ms).  A system
+// whose device histogram the caller can write to is copied at its own first
+// read only.
 int fetch_histogram(Context *c, System &s)
 {
     if (!c->ran) return fail(c, MUCAL_ERR_NOT_READY, "no iteration has been run");
+    s.hist_ahead = false;
     if (s.hist_on_host) return MUCAL_OK;
     CUDA_TRY(c, cudaMemcpyAsync(c->h_H, c->d_H, (c->h_words + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -710,9 +715,10 @@ int fetch_histogram(Context *c, System &s)
                                         "(flag %u); the iteration's results are not valid", err);
     }
     for (auto &q : c->sys) {
-        if (q.hist_on_host) continue;
+        if (q.hist_on_host || (&q != &s && q.hist_shared)) continue;
         std::memcpy(q.H.data(), c->h_H + q.h_off, q.H.size() * sizeof(int64_t));
         q.hist_on_host = true;
+        q.hist_ahead = &q != &s;
     }
     return MUCAL_OK;
 }
@@ -1139,7 +1145,7 @@ int mucal_run_iteration(void *ctx, int64_t sweeps, uint32_t iteration)
         CUDA_TRY(c, cudaEventRecord(c->ev_it1, c->stream));
     }
     for (auto &s : c->sys) {
-        s.hist_on_host = false;
+        s.hist_on_host = s.hist_ahead = false;
         s.last_attempts = (uint64_t)sweeps * (uint64_t)s.p.N * (uint64_t)s.p.n_walkers;
         s.lnW_run = s.lnW;
     }
@@ -1205,6 +1211,7 @@ int mucal_set_histogram(void *ctx, int32_t sys, const int64_t *H, int32_t n_bins
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     std::copy(H, H + n_bins, s.H.begin());
     s.hist_on_host = true;
+    s.hist_ahead = false;
     return MUCAL_OK;
 }
 
@@ -1344,7 +1351,10 @@ int mucal_histogram_device_ptr(void *ctx, int32_t sys, void **dptr)
     int rc = check_sys(c, sys);
     if (rc != MUCAL_OK) return rc;
     if (!dptr) return fail(c, MUCAL_ERR_INVALID_ARG, "dptr is NULL");
-    *dptr = c->sys[sys].p.H;
+    System &s = c->sys[sys];
+    s.hist_shared = true;
+    if (s.hist_ahead) s.hist_on_host = s.hist_ahead = false;
+    *dptr = s.p.H;
     return MUCAL_OK;
 }
 

@@ -807,3 +807,40 @@ def test_default_shape_bit_exact(desc):
         np.testing.assert_array_equal(mc.histogram(0), hist.sum(axis=0))
         for w in range(W):
             _assert_walker_equal(mc, 0, w, S[w], occ[w], E[w])
+
+
+# ------------------------------------------------- histograms on the device
+
+def _device_view(mc, k):
+    import torch
+
+    class Rows:
+        __cuda_array_interface__ = {"data": (m.mucal_histogram_device_ptr(mc.ctx, k), False), "typestr": "<i8",
+                                    "shape": (mc.info[k]["n_bins"],), "version": 3}
+    return torch.as_tensor(Rows(), device="cuda")
+
+
+@pytest.mark.parametrize("late", [False, True])
+def test_histograms_changed_on_the_device_system_by_system(late):
+    """A change of a system's device histogram counts in that system's first
+    read, also after another system has been read; the pointers are taken
+    before any read or (late) after one."""
+    import torch
+    systems = [(2, 16, 32, 64, 0, 0, 0), (2, 12, 20, 40, 0, 0, 100), (3, 6, 25, 30, 0, 0, 200)]
+    with m.Mucal(systems) as mc, m.Mucal(systems) as ref:
+        views = {} if late else {k: _device_view(mc, k) for k in range(3)}
+        for it in range(2):
+            mc.run_iteration(5, it)
+            ref.run_iteration(5, it)
+            for k in range(3):
+                want = ref.histogram(k)
+                if k > 0:
+                    views.setdefault(k, _device_view(mc, k))
+                    torch.cuda.synchronize()
+                    views[k] += k
+                    torch.cuda.synchronize()
+                    want = want + k
+                np.testing.assert_array_equal(mc.histogram(k), want)
+                lnW, _ = mc.update_weights(k)
+                ref.set_histogram(k, want)
+                np.testing.assert_array_equal(lnW, ref.update_weights(k)[0])
