@@ -442,9 +442,11 @@ int mfail(Mlp *m, int code, const std::string &msg)
 #define MLP_TRY(m, call)                                                                        \
     do {                                                                                        \
         cudaError_t e_ = (call);                                                                \
-        if (e_ != cudaSuccess)                                                                  \
+        if (e_ != cudaSuccess) {                                                                \
+            cudaGetLastError();     /* not for the check behind the next launch */              \
             return mfail((m), e_ == cudaErrorMemoryAllocation ? MUCAL_ERR_OOM : MUCAL_ERR_CUDA, \
                          std::string(#call ": ") + cudaGetErrorString(e_));                     \
+        }                                                                                       \
     } while (0)
 
 int ensure_capacity(Mlp *m, int64_t B)
@@ -571,6 +573,7 @@ int mucal_mlp_create(void **out, const float *params, int64_t n, void *cuda_stre
     Mlp *m = new Mlp();
     auto bail = [&](int code) {
         g_mlp_err = m->err;
+        cudaGetLastError();
         cudaFree(m->w); cudaFree(m->grad); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->wq); cudaFree(m->w2t);
         cudaFree(m->loss);
         if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);

@@ -110,12 +110,16 @@ int fail(Context *c, int code, const char *fmt, ...)
     return code;
 }
 
+// (a reported error is taken back from the runtime, which would hand it to the
+// check behind the next launch)
 #define CUDA_TRY(ctx, call)                                                                  \
     do {                                                                                     \
         cudaError_t e_ = (call);                                                             \
-        if (e_ != cudaSuccess)                                                               \
+        if (e_ != cudaSuccess) {                                                             \
+            cudaGetLastError();                                                              \
             return fail((ctx), e_ == cudaErrorMemoryAllocation ? MUCAL_ERR_OOM : MUCAL_ERR_CUDA, \
                         "%s: %s (%s:%d)", #call, cudaGetErrorString(e_), __FILE__, __LINE__); \
+        }                                                                                    \
     } while (0)
 
 // ---------------------------------------------------------------------------
@@ -453,6 +457,7 @@ int build_work(Context *c, const LaunchShape &sh)
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_sys, hp.data(), hp.size() * sizeof(SysParams), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         cudaFree(d_work);
         cudaFree(d_reduce);
         cudaFree(d_hist);
@@ -861,6 +866,7 @@ int mucal_init_systems(void **out, const mucal_system_desc *sys, int32_t n_sys, 
     int rc = MUCAL_OK;
     auto bail = [&](int code) {
         if (c->err.size()) g_init_error = c->err;
+        cudaGetLastError();
         destroy_context(c);
         return code;
     };

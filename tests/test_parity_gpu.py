@@ -844,3 +844,31 @@ def test_histograms_changed_on_the_device_system_by_system(late):
                 lnW, _ = mc.update_weights(k)
                 ref.set_histogram(k, want)
                 np.testing.assert_array_equal(lnW, ref.update_weights(k)[0])
+
+
+def test_failed_shape_change_leaves_the_context_usable():
+    """A shape whose histogram rows do not fit on the device is refused, and
+    the next iteration runs in the shape before as if nothing had been asked."""
+    import torch
+    desc = (3, 20, 4000, 16384, 0, 0, 0)           # rows of one walker each: 1.6 GB
+    big = dict(kernel=m.MUCAL_KERNEL_GROUP, lanes_per_walker=32, walkers_per_block=1)
+    with m.Mucal([desc]) as mc, m.Mucal([desc]) as ref:
+        shape = mc.launch()
+        mc.run_iteration(1, 0)
+        ref.run_iteration(1, 0)
+        torch.cuda.synchronize()
+        rest = torch.empty(max(0, torch.cuda.mem_get_info()[0] - (1 << 30)), dtype=torch.uint8, device="cuda")
+        try:
+            with pytest.raises(m.MucalError):
+                mc.set_launch(**big)
+        finally:
+            del rest
+            torch.cuda.empty_cache()
+        assert mc.launch() == shape
+        mc.run_iteration(1, 1)
+        ref.run_iteration(1, 1)
+        np.testing.assert_array_equal(mc.histogram(0), ref.histogram(0))
+        mc.set_launch(**big)                        # and in the new one, now that there is room
+        mc.run_iteration(1, 2)
+        ref.run_iteration(1, 2)
+        np.testing.assert_array_equal(mc.histogram(0), ref.histogram(0))
