@@ -350,8 +350,9 @@ cudaError_t droplet_plan(const SysParams &p, DropletPlan *plan)
     plan->shared = need + static_bytes <= (size_t)optin;
     if (plan->shared) {
         plan->smem = need;
+        // (as much as there is, not this lattice's need: plans of other lattices are kept)
         e = cudaFuncSetAttribute(droplet_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)need);
+                                 optin - (int)static_bytes);
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, droplet_kernel<true>,
                                                               kDropThreads, need);

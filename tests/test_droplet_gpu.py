@@ -225,3 +225,14 @@ def test_production_curve_against_enumeration():
         assert row["specific_heat_per_site"] == pytest.approx(cv, rel=0.05, abs=2e-3), row
         assert row["mean_V_D"] == pytest.approx((w * D).sum() / w.sum(), abs=0.05), row
         assert row["mean_E_ising"] == pytest.approx(4 * (row["mean_E"] - muca.ising_constant(d, L, N)))
+
+
+def test_droplets_of_two_contexts_in_turn():
+    """Dense lattices whose parents fit a block's shared memory but not the
+    tables by rank: a context's second measurement after a smaller lattice's."""
+    a, b = (2, 230, 38000, 2, 0, 0, 1), (2, 225, 37500, 2, 0, 0, 2)
+    with m.Mucal([a]) as ca, m.Mucal([b]) as cb:
+        for c, (d, L, N, W, _, _, seed) in ((ca, a), (cb, b), (ca, a)):
+            c.measure_droplets()
+            _, occ, _ = chain.init_walkers(d, L, N, W, seed)
+            assert c.largest_droplets(0).tolist() == [chain.largest_droplet(d, L, occ[w]) for w in range(W)]
