@@ -611,6 +611,10 @@ int default_lanes(long long r, double N)
 // against several commits): 2D L = 10, N = 8, 64 walkers 0.63 and 0.42 against
 // 0.77 and 0.49; 2D L = 22, N = 12, 64 walkers 0.59 and 0.51 against 0.53 and
 // 0.45, 3000 walkers 0.73 and 0.62 against 0.52 and 0.48 (4 lanes).
+// Lattices whose bitsets stay in global memory (2D L = 1400) have a few
+// particles far apart, and several commits pay from 8 on (3 and 512 walkers,
+// 4000 attempts): N = 4 1.43 and 2.32 against 1.98 and 2.54, N = 8 1.36 and 2.45
+// against 1.36 and 1.81, N = 11 1.32 and 2.48 against 1.16 and 1.56.
 mucal_launch_config default_launch(Context *c)
 {
     long long total = 0;
@@ -657,8 +661,12 @@ mucal_launch_config default_launch(Context *c)
     long long cap = most(MUCAL_KERNEL_GROUP);
     if (cap < 1) {                           // bitsets in global memory
         def.bits_in_smem = 0;
-        def.lanes_per_walker = default_lanes(need, N);
-        if (def.lanes_per_walker == 4) def.lanes_per_walker = 8;
+        if (N < 8) {
+            def.multi_commit = 0;
+            def.thr_window = 1;
+        } else {
+            def.lanes_per_walker = std::max(8, default_lanes(need, N));
+        }
         return def;
     }
     if (plain_fits(MUCAL_KERNEL_FIELD)) {

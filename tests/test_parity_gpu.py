@@ -872,3 +872,16 @@ def test_failed_shape_change_leaves_the_context_usable():
         mc.run_iteration(1, 2)
         ref.run_iteration(1, 2)
         np.testing.assert_array_equal(mc.histogram(0), ref.histogram(0))
+
+
+def test_default_shape_of_few_particles_on_a_large_lattice():
+    """One commit per round below 8 particles where no walker's bitset fits a
+    block."""
+    for N, several in ((7, 0), (8, 1)):
+        with m.Mucal([(2, 1400, N, 3, 0, 0, 4)]) as mc:
+            assert mc.launch()["multi_commit"] == several and mc.launch()["bits_in_smem"] == 0
+            S, occ, E = _oracle_states(2, 1400, N, 3, 4)
+            T = chain.thresholds(2, -2 * N, 0, np.zeros(2 * N + 1))
+            mc.run_iteration(9, 0)
+            hist, _ = chain.run_walkers(2, 1400, N, 4, 0, 9 * N, -2 * N, 0, T, S, occ, E)
+            np.testing.assert_array_equal(mc.histogram(0), hist.sum(axis=0))
