@@ -580,9 +580,16 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
 // 0.27, 0.37 and 0.18 (0.46, 0.17); 2D L = 40, N = 100, r = 60: 0.83 and 0.46,
 // 0.79 and 0.38 (1.03, 0.39); 2D L = 40, N = 60, r = 1, 16 lanes: 0.55 and 0.19
 // (0.81, 0.26).
-int default_lanes(long long r, double N)
+//
+// More than 64 walkers beside each other have registers at 4 lanes only (512
+// threads of 128).  One system in one wave at 4 lanes against two waves at 8 (and
+// 32 walkers a block at 16, and one commit per round), at acceptance 1, 0.3 and
+// 0.03: 2D L = 26, N = 80, r = 100 1.41, 0.97 and 0.59 ms against 1.81, 1.42 and
+// 0.63 (4.67, 2.89 and 0.77; 1.92, 1.19 and 0.65); 2D L = 58, N = 400, r = 72
+// 1.31, 0.77 and 0.53 against 1.07, 0.94 and 0.56.
+int default_lanes(long long r, double N, bool one)
 {
-    if ((N < 48 && r >= 12) || (N < 64 && r > 48)) return 4;
+    if ((N < 48 && r >= 12) || (N < 64 && r > 48) || (one && r > 64)) return 4;
     if (N >= 2500 && r <= 7) return 32;
     if ((N >= 1000 && r <= 24) || (N >= 60 && r <= 4)) return 16;
     return 8;
@@ -665,7 +672,7 @@ mucal_launch_config default_launch(Context *c)
             def.multi_commit = 0;
             def.thr_window = 1;
         } else {
-            def.lanes_per_walker = std::max(8, default_lanes(need, N));
+            def.lanes_per_walker = std::max(8, default_lanes(need, N, true));
         }
         return def;
     }
@@ -683,20 +690,33 @@ mucal_launch_config default_launch(Context *c)
         return def;
     }
     const bool one = c->sys.size() == 1;
-    const long long waves = (need + cap - 1) / cap;
-    const long long r = one ? (need + waves - 1) / waves : std::min(need, cap);
-    const long long want = one ? r : (fits(def.kernel, 8) == 2 ? 8 : 4);
-    // whole warps: blocks of 32 / lanes walkers and multiples; wider groups
-    // come in finer blocks
-    for (int lanes = default_lanes(r, N);; lanes *= 2) {
+    // walkers per SM of one of the fewest equal waves, `room` walkers at a time
+    auto wave = [&](long long room) {
+        const long long waves = (need + room - 1) / room;
+        return (need + waves - 1) / waves;
+    };
+    const long long r = one ? wave(cap) : std::min(need, cap);
+    long long want = one ? r : (fits(def.kernel, 8) == 2 ? 8 : 4);
+    int lanes = default_lanes(r, N, one);
+    // whole warps: blocks of 32 / lanes walkers and multiples, of at most 512 threads
+    for (;;) {
         const long long step = 32 / lanes;
         const long long top = std::min<long long>(cap, 512 / lanes) / step * step;
         const long long w = (want + step - 1) / step * step;
-        def.lanes_per_walker = lanes;
-        def.walkers_per_block = (int)std::min(w, top);
-        if (top >= step && (w <= top || lanes >= 16)) break;    // (at 32 lanes always)
+        if (top >= step && w <= top) {
+            def.lanes_per_walker = lanes;
+            def.walkers_per_block = (int)w;
+            return def;
+        }
+        // wider groups come in finer blocks; else more waves
+        const long long fine = step / 2, finer = std::min<long long>(cap, 256 / lanes);
+        if (top < step || (fine > 0 && (want + fine - 1) / fine * fine <= finer)) {
+            lanes *= 2;
+            continue;
+        }
+        want = one ? wave(top) : top;
+        lanes = std::max(lanes, default_lanes(want, N, one));
     }
-    return def;
 }
 
 Context *as_ctx(void *p) { return static_cast<Context *>(p); }

@@ -885,3 +885,28 @@ def test_default_shape_of_few_particles_on_a_large_lattice():
             mc.run_iteration(9, 0)
             hist, _ = chain.run_walkers(2, 1400, N, 4, 0, 9 * N, -2 * N, 0, T, S, occ, E)
             np.testing.assert_array_equal(mc.histogram(0), hist.sum(axis=0))
+
+
+@pytest.mark.parametrize("d,L,N,r,lanes,wpb", [
+    (2, 30, 100, 100, 4, 104),       # more walkers per SM than 8 lanes have registers for
+    (2, 14, 30, 65, 4, 72),
+    (2, 30, 100, 64, 8, 64),
+    (2, 200, 3500, 33, 16, 18),      # 35 fit, whole warps hold 32: two waves
+])
+def test_default_shape_of_many_walkers(d, L, N, r, lanes, wpb):
+    """Blocks of whole warps and at most 512 threads hold an SM's walkers in as
+    few equal waves as they can."""
+    import torch
+    W, seed = r * torch.cuda.get_device_properties(0).multi_processor_count - 3, 17
+    with m.Mucal([(d, L, N, W, 0, 0, seed)]) as mc:
+        launch = mc.launch()
+        assert (launch["lanes_per_walker"], launch["walkers_per_block"]) == (lanes, wpb)
+        assert launch["multi_commit"] == 1
+        mc.run_iteration(2, 0)
+        assert mc.histogram(0).sum() == W * 2 * N
+        pick = [0, wpb - 1, wpb, W - 1]
+        S, occ, E = _oracle_states(d, L, N, W, seed, pick)
+        T = chain.thresholds(d, -d * N, 0, np.zeros(d * N + 1))
+        chain.run_walkers(d, L, N, seed, 0, 2 * N, -d * N, 0, T, S, occ, E, walkers=pick)
+        for q, w in enumerate(pick):
+            _assert_walker_equal(mc, 0, w, S[q], occ[q], E[q])
