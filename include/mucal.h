@@ -116,8 +116,9 @@ typedef struct mucal_system_desc {
 
 /* A new context has a shape chosen from its systems' sizes and walkers: several
    commits per round from 12 particles up (from 8 where a lattice's bitset does
-   not fit a block's shared memory), one below; as many walkers side by side as
-   there are or as shared memory holds.  The defaults below are those of a
+   not fit a block's shared memory), one below and where lattices are so small and
+   dense that attempts mostly get in each other's way; as many walkers side by side
+   as there are or as shared memory holds.  The defaults below are those of a
    configuration that names only some fields. */
 typedef struct mucal_launch_config {
     int32_t kernel;            /* MUCAL_KERNEL_THREAD, _GROUP or _FIELD */

@@ -574,12 +574,16 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
 // 13.0 / -; 2D L = 64, N = 410, r = 1: 4.29 / 2.74 / 2.28 / 2.79, r = 10: 4.35 /
 // 2.80 / 3.05 / 7.3; 3D L = 8, N = 56, r = 56: 1.44 / 1.98 / 5.2 / -.
 // Narrow windows pay while moves are accepted; where they are refused, wide
-// ones pass over more at a time.  At acceptance 0.8 and 0.04 (with one commit
-// per round, 8 lanes, behind it): 2D L = 14, N = 24, r = 20: 4 lanes 0.51 and
-// 0.31, 8 lanes 0.71 and 0.22 (0.68, 0.22); 2D L = 20, N = 20, r = 7: 0.39 and
-// 0.27, 0.37 and 0.18 (0.46, 0.17); 2D L = 40, N = 100, r = 60: 0.83 and 0.46,
-// 0.79 and 0.38 (1.03, 0.39); 2D L = 40, N = 60, r = 1, 16 lanes: 0.55 and 0.19
-// (0.81, 0.26).
+// ones pass over more at a time.  Only where more than 48 walkers of few
+// particles share an SM, so that instructions bound them, are 4 lanes no loss
+// against one commit per round (8 lanes) at any acceptance.  The time of one
+// commit per round over that of several at 4 and at 8 lanes, at acceptance 1, 0.35,
+// 0.15 and 0.05: 2D L = 12, N = 18, r = 16 1.09, 0.86, 0.69, 0.62 and 0.95, 0.93,
+// 0.90, 1.00; r = 32 1.26, 1.01, 0.82, 0.74 and 0.82, 0.84, 0.86, 1.02; r = 56 1.40,
+// 1.12, 0.95, 0.95 and 0.76, 0.76, 0.80, 1.04; 2D L = 34, N = 47, r = 16 (acceptance
+// 1, 0.33, 0.09, 0.01) 1.30, 0.91, 0.68, 0.61 and 1.58, 1.26, 1.02, 1.02; r = 56 1.59,
+// 1.15, 0.95, 0.99 and 1.23, 0.97, 0.97, 1.23.  At 16 lanes 2D L = 45, N = 80, r = 4
+// gains 2.01, 1.40, 1.21 and 1.60.
 //
 // More than 64 walkers beside each other have registers at 4 lanes only (512
 // threads of 128).  One system in one wave at 4 lanes against two waves at 8 (and
@@ -589,7 +593,7 @@ int apply_launch_config(Context *c, const mucal_launch_config &cfg)
 // 1.31, 0.77 and 0.53 against 1.07, 0.94 and 0.56.
 int default_lanes(long long r, double N, bool one)
 {
-    if ((N < 48 && r >= 12) || (N < 64 && r > 48) || (one && r > 64)) return 4;
+    if ((N < 64 && r > 48) || (one && r > 64)) return 4;
     if (N >= 2500 && r <= 7) return 32;
     if ((N >= 1000 && r <= 24) || (N >= 60 && r <= 4)) return 16;
     return 8;
@@ -613,11 +617,18 @@ int default_lanes(long long r, double N, bool one)
 // resident walker: 2D L = 64 3.24 (bitsets) -> 3.11, but five 2D systems of
 // L = 61 to 97, 5120 walkers, 50 sweeps 1.06 (bitsets) against 1.9.
 //
-// Below 12 particles nearly every window holds a conflict, and the rounds with
-// one commit are faster (8 lanes, ms at a high and a middle acceptance, one
-// against several commits): 2D L = 10, N = 8, 64 walkers 0.63 and 0.42 against
-// 0.77 and 0.49; 2D L = 22, N = 12, 64 walkers 0.59 and 0.51 against 0.53 and
-// 0.45, 3000 walkers 0.73 and 0.62 against 0.52 and 0.48 (4 lanes).
+// Below 12 particles, and on small dense lattices above, nearly every window
+// holds a conflict, and the rounds with one commit (8 lanes, 16 walkers a block)
+// are the faster ones.  What counts is the chance that two attempts touch (a
+// list slot in common, 1 / N and 1 / (V - N), or sites next to each other, 8 d /
+// V) and whether latency (few walkers per SM) or instructions (many) bound the
+// rounds.  The time of one commit per round over that of several at 8 lanes, the
+// worst and best over acceptances from 1 to 0.001: at r = 11 touch 0.25 (2D
+// L = 10, N = 12) 0.82 to 1.26, 0.21 (L = 11, N = 14) 0.88 to 1.26, 0.17 (L = 12,
+// N = 18) 0.89 to 1.26, 0.13 (L = 14, N = 24) 0.94 to 1.31, 0.07 (L = 24, N = 24)
+// 0.99 to 1.35; at r = 32 touch 0.17 0.82 to 1.34, 0.10 (L = 16, N = 30) 0.90 to
+// 1.41, at r = 40 0.86 to 1.47, 0.09 (L = 17, N = 36) 0.89 to 1.47, 0.06 (L = 20,
+// N = 47) 0.90 to 1.48, 0.05 (L = 30, N = 36) 0.95 to 1.40.
 // Lattices whose bitsets stay in global memory (2D L = 1400) have a few
 // particles far apart, and several commits pay from 8 on (3 and 512 walkers,
 // 4000 attempts): N = 4 1.43 and 2.32 against 1.98 and 2.54, N = 8 1.36 and 2.45
@@ -625,13 +636,16 @@ int default_lanes(long long r, double N, bool one)
 mucal_launch_config default_launch(Context *c)
 {
     long long total = 0;
-    double work = 0.0, work_n = 0.0;
+    double work = 0.0, work_n = 0.0, work_t = 0.0;
     for (auto &s : c->sys) {
+        const double n = s.p.N, v = s.p.V, w = s.p.n_walkers * n;
         total += s.p.n_walkers;
-        work += (double)s.p.n_walkers * s.p.N;
-        work_n += (double)s.p.n_walkers * s.p.N * s.p.N;
+        work += w;
+        work_n += w * n;
+        work_t += w * (1.0 / n + 1.0 / (v - n) + 8.0 * s.p.d / v);
     }
     const double N = work_n / work;     // particles of the system an average attempt belongs to
+    const double touch = work_t / work; // chance that two attempts touch
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     const long long need = (total + sms - 1) / sms;     // walkers per SM
@@ -683,12 +697,6 @@ mucal_launch_config default_launch(Context *c)
             cap = f;
         }
     }
-    if (N < 12) {
-        def.multi_commit = 0;
-        def.thr_window = 1;
-        if (!plain_fits(def.kernel)) def.bits_in_smem = 0;
-        return def;
-    }
     const bool one = c->sys.size() == 1;
     // walkers per SM of one of the fewest equal waves, `room` walkers at a time
     auto wave = [&](long long room) {
@@ -696,6 +704,12 @@ mucal_launch_config default_launch(Context *c)
         return (need + waves - 1) / waves;
     };
     const long long r = one ? wave(cap) : std::min(need, cap);
+    if (N < 12 || (r <= 16 && touch > 0.175) || (r > 16 && r <= 48 && touch > 0.08)) {
+        def.multi_commit = 0;
+        def.thr_window = 1;
+        if (!plain_fits(def.kernel)) def.bits_in_smem = 0;
+        return def;
+    }
     long long want = one ? r : (fits(def.kernel, 8) == 2 ? 8 : 4);
     int lanes = default_lanes(r, N, one);
     // whole warps: blocks of 32 / lanes walkers and multiples, of at most 512 threads

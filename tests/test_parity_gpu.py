@@ -910,3 +910,28 @@ def test_default_shape_of_many_walkers(d, L, N, r, lanes, wpb):
         chain.run_walkers(d, L, N, seed, 0, 2 * N, -d * N, 0, T, S, occ, E, walkers=pick)
         for q, w in enumerate(pick):
             _assert_walker_equal(mc, 0, w, S[q], occ[q], E[q])
+
+
+@pytest.mark.parametrize("d,L,N,r,lanes,several", [
+    (2, 10, 12, 2, 8, 0),            # small and dense: attempts touch with a chance of 0.25
+    (2, 14, 24, 14, 8, 1),           # 0.13, few walkers per SM
+    (2, 14, 24, 20, 8, 0),           # and many
+    (2, 34, 47, 20, 8, 1),           # 0.04
+    (3, 9, 40, 60, 4, 1),
+])
+def test_default_shape_of_few_particles(d, L, N, r, lanes, several):
+    """One commit per round where attempts mostly touch, 4 lanes only where
+    many walkers share an SM."""
+    import torch
+    W, seed = r * torch.cuda.get_device_properties(0).multi_processor_count - 3, 5
+    with m.Mucal([(d, L, N, W, 0, 0, seed)]) as mc:
+        launch = mc.launch()
+        assert (launch["lanes_per_walker"], launch["multi_commit"]) == (lanes, several)
+        mc.run_iteration(3, 0)
+        assert mc.histogram(0).sum() == W * 3 * N
+        pick = [0, W // 2, W - 1]
+        S, occ, E = _oracle_states(d, L, N, W, seed, pick)
+        T = chain.thresholds(d, -d * N, 0, np.zeros(d * N + 1))
+        chain.run_walkers(d, L, N, seed, 0, 3 * N, -d * N, 0, T, S, occ, E, walkers=pick)
+        for q, w in enumerate(pick):
+            _assert_walker_equal(mc, 0, w, S[q], occ[q], E[q])
