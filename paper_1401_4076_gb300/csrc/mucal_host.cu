@@ -8,6 +8,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -610,7 +611,11 @@ int default_lanes(long long r, double N, bool one)
 // sweeps 15.9 -> 12.4 (28, two waves).  Several systems: small blocks, which
 // pack their uneven bitsets and lengths best (the 27-system batch, 5 sweeps:
 // 4 walkers 9.2, 14 walkers 10.9), of 8 walkers where a block stages the
-// table.
+// table, or of 16, or with bitsets for count fields, where these make fewer waves
+// with a table in every block: five systems of 3D L = 14, N = 300, 540 walkers, 10
+// sweeps, 8 -> 16 walkers at acceptance 1, 0.1 and 0.01 1.24, 0.85 and 0.97 times the
+// speed of one commit per round -> 1.73, 1.28 and 1.54; six of 3D L = 23, N = 300, 280
+// walkers, fields -> bitsets 1.45, 0.85 and 0.90 -> 2.88, 1.59 and 1.72.
 //
 // Count fields (two byte loads per attempt instead of 4d words, 4d more
 // atomics per commit) where they fit 16 walkers to a block and do not cost a
@@ -646,8 +651,10 @@ mucal_launch_config default_launch(Context *c)
     }
     const double N = work_n / work;     // particles of the system an average attempt belongs to
     const double touch = work_t / work; // chance that two attempts touch
-    int sms = 1;
+    int sms = 1, sm_smem = 0, reserved = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device);
+    cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, c->device);
     const long long need = (total + sms - 1) / sms;     // walkers per SM
     // whether w walkers fit a block: 0 no, 1 with row windows, 2 with the table
     auto fits = [&](int kernel, int w) {
@@ -710,8 +717,40 @@ mucal_launch_config default_launch(Context *c)
         if (!plain_fits(def.kernel)) def.bits_in_smem = 0;
         return def;
     }
-    long long want = one ? r : (fits(def.kernel, 8) == 2 ? 8 : 4);
     int lanes = default_lanes(r, N, one);
+    long long want = r;
+    if (!one) {
+        // waves of blocks of w walkers that stage the table (0: it does not fit)
+        auto waves = [&](int kernel, int w) -> long long {
+            if (fits(kernel, w) != 2) return 0;
+            LaunchShape sh{};
+            sh.kernel = kernel;
+            sh.walkers_per_block = w;
+            sh.bits_in_smem = sh.thr_in_smem = 1;
+            size_t smem = 0;
+            long long blocks = 0;
+            for (auto &s : c->sys) {
+                smem = std::max(smem, smem_for(sh, s.p));
+                blocks += (s.p.n_walkers + w - 1) / w;
+            }
+            const int threads = std::max(32, w * lanes);
+            const long long per_sm = std::min<long long>({sm_smem / (int)(smem + mucal::kWalkerStaticSmem + reserved),
+                                                          512 / threads, 32});
+            return (blocks + sms * per_sm - 1) / (sms * per_sm);
+        };
+        long long least = waves(def.kernel, 8);
+        want = least ? 8 : 4;
+        const std::pair<int, int> others[] = {
+            {def.kernel, 16}, {MUCAL_KERNEL_GROUP, 8}, {MUCAL_KERNEL_GROUP, 16}};
+        for (auto &o : others) {
+            const long long n = least > 1 ? waves(o.first, o.second) : 0;
+            if (n == 0 || n >= least) continue;
+            least = n;
+            def.kernel = o.first;
+            want = o.second;
+        }
+        cap = most(def.kernel);
+    }
     // whole warps: blocks of 32 / lanes walkers and multiples, of at most 512 threads
     for (;;) {
         const long long step = 32 / lanes;

@@ -935,3 +935,28 @@ def test_default_shape_of_few_particles(d, L, N, r, lanes, several):
         chain.run_walkers(d, L, N, seed, 0, 3 * N, -d * N, 0, T, S, occ, E, walkers=pick)
         for q, w in enumerate(pick):
             _assert_walker_equal(mc, 0, w, S[q], occ[q], E[q])
+
+
+@pytest.mark.parametrize("desc,systems,kernel,wpb", [
+    ((3, 14, 300, 540), 5, m.MUCAL_KERNEL_FIELD, 16),    # two blocks an SM, whatever they hold
+    ((3, 23, 300, 280), 6, m.MUCAL_KERNEL_GROUP, 8),     # one block of count fields an SM
+    ((3, 21, 100, 256), 8, m.MUCAL_KERNEL_FIELD, 8),     # one wave as it is
+])
+def test_default_shape_of_several_systems(desc, systems, kernel, wpb):
+    """Blocks of several systems that stage a table each make as few waves as
+    they can."""
+    import torch
+    d, L, N, W = desc
+    W = W * torch.cuda.get_device_properties(0).multi_processor_count // 152
+    with m.Mucal([(d, L, N, W, 0, 0, 10 ** 6 * i) for i in range(systems)]) as mc:
+        launch = mc.launch()
+        assert (launch["kernel"], launch["walkers_per_block"]) == (kernel, wpb)
+        assert (launch["lanes_per_walker"], launch["multi_commit"]) == (8, 1)
+        mc.run_iteration(1, 0)
+        for i in (0, systems - 1):
+            assert mc.histogram(i).sum() == W * N
+            S, occ, E = _oracle_states(d, L, N, W, 10 ** 6 * i, [0, W - 1])
+            T = chain.thresholds(d, -d * N, 0, np.zeros(d * N + 1))
+            chain.run_walkers(d, L, N, 10 ** 6 * i, 0, N, -d * N, 0, T, S, occ, E, walkers=[0, W - 1])
+            for q, w in enumerate((0, W - 1)):
+                _assert_walker_equal(mc, i, w, S[q], occ[q], E[q])
