@@ -634,6 +634,11 @@ int default_lanes(long long r, double N, bool one)
 // 0.99 to 1.35; at r = 32 touch 0.17 0.82 to 1.34, 0.10 (L = 16, N = 30) 0.90 to
 // 1.41, at r = 40 0.86 to 1.47, 0.09 (L = 17, N = 36) 0.89 to 1.47, 0.06 (L = 20,
 // N = 47) 0.90 to 1.48, 0.05 (L = 30, N = 36) 0.95 to 1.40.
+// They take count fields where 48 walkers, or all there are, are resident on an SM
+// in blocks of 16 (ms, fields and bitsets): 2D L = 60, N = 8, 48 a wave, 108 per SM
+// 3.64 and 4.07; 2D L = 80, N = 10, 32 a wave, 30 per SM 1.20 and 1.46, 48 2.11 and
+// 1.87, 64 2.38 and 2.34, 100 4.35 and 3.98; 2D L = 100, N = 11, 16 a wave, 48 per SM
+// 2.85 and 1.85.
 // Lattices whose bitsets stay in global memory (2D L = 1400) have a few
 // particles far apart, and several commits pay from 8 on (3 and 512 walkers,
 // 4000 attempts): N = 4 1.43 and 2.32 against 1.98 and 2.54, N = 8 1.36 and 2.45
@@ -671,6 +676,18 @@ mucal_launch_config default_launch(Context *c)
         }
         return 0;
     };
+    // shared memory of a block of w walkers, with the table where it fits
+    auto block_smem = [&](int kernel, int w) {
+        LaunchShape sh{};
+        sh.kernel = kernel;
+        sh.walkers_per_block = w;
+        sh.bits_in_smem = sh.scan_window = 1;
+        sh.thr_in_smem = fits(kernel, w) == 2 ? 1 : 0;
+        size_t smem = 0;
+        for (auto &s : c->sys) smem = std::max(smem, smem_for(sh, s.p));
+        return (int)smem;
+    };
+    const int overhead = mucal::kWalkerStaticSmem + reserved;    // beside it
     auto plain_fits = [&](int kernel) {      // without table and windows
         LaunchShape sh{};
         sh.kernel = kernel;
@@ -714,6 +731,11 @@ mucal_launch_config default_launch(Context *c)
     if (N < 12 || (r <= 16 && touch > 0.175) || (r > 16 && r <= 48 && touch > 0.08)) {
         def.multi_commit = 0;
         def.thr_window = 1;
+        def.kernel = MUCAL_KERNEL_GROUP;
+        if (plain_fits(MUCAL_KERNEL_FIELD)) {
+            const long long resident = 16 * (sm_smem / (block_smem(MUCAL_KERNEL_FIELD, 16) + reserved + 64));
+            if (resident >= std::min<long long>(need, 48)) def.kernel = MUCAL_KERNEL_FIELD;
+        }
         if (!plain_fits(def.kernel)) def.bits_in_smem = 0;
         return def;
     }
@@ -723,18 +745,10 @@ mucal_launch_config default_launch(Context *c)
         // waves of blocks of w walkers that stage the table (0: it does not fit)
         auto waves = [&](int kernel, int w) -> long long {
             if (fits(kernel, w) != 2) return 0;
-            LaunchShape sh{};
-            sh.kernel = kernel;
-            sh.walkers_per_block = w;
-            sh.bits_in_smem = sh.thr_in_smem = 1;
-            size_t smem = 0;
             long long blocks = 0;
-            for (auto &s : c->sys) {
-                smem = std::max(smem, smem_for(sh, s.p));
-                blocks += (s.p.n_walkers + w - 1) / w;
-            }
+            for (auto &s : c->sys) blocks += (s.p.n_walkers + w - 1) / w;
             const int threads = std::max(32, w * lanes);
-            const long long per_sm = std::min<long long>({sm_smem / (int)(smem + mucal::kWalkerStaticSmem + reserved),
+            const long long per_sm = std::min<long long>({sm_smem / (block_smem(kernel, w) + overhead),
                                                           512 / threads, 32});
             return (blocks + sms * per_sm - 1) / (sms * per_sm);
         };

@@ -960,3 +960,24 @@ def test_default_shape_of_several_systems(desc, systems, kernel, wpb):
             chain.run_walkers(d, L, N, 10 ** 6 * i, 0, N, -d * N, 0, T, S, occ, E, walkers=[0, W - 1])
             for q, w in enumerate((0, W - 1)):
                 _assert_walker_equal(mc, i, w, S[q], occ[q], E[q])
+
+
+@pytest.mark.parametrize("L,N,r,kernel", [
+    (60, 8, 70, m.MUCAL_KERNEL_FIELD),     # 48 walkers of count fields an SM
+    (80, 10, 32, m.MUCAL_KERNEL_FIELD),    # 32, all there are
+    (80, 10, 33, m.MUCAL_KERNEL_GROUP),
+    (100, 11, 33, m.MUCAL_KERNEL_GROUP),   # 16
+])
+def test_default_kernel_of_one_commit_rounds(L, N, r, kernel):
+    import torch
+    W = r * torch.cuda.get_device_properties(0).multi_processor_count
+    with m.Mucal([(2, L, N, W, 0, 0, 9)]) as mc:
+        launch = mc.launch()
+        assert (launch["kernel"], launch["multi_commit"], launch["walkers_per_block"]) == (kernel, 0, 16)
+        mc.run_iteration(5, 0)
+        assert mc.histogram(0).sum() == W * 5 * N
+        S, occ, E = _oracle_states(2, L, N, 40, 9)
+        T = chain.thresholds(2, -2 * N, 0, np.zeros(2 * N + 1))
+        chain.run_walkers(2, L, N, 9, 0, 5 * N, -2 * N, 0, T, S, occ, E)
+        for w in (0, 17, 39):
+            _assert_walker_equal(mc, 0, w, S[w], occ[w], E[w])
