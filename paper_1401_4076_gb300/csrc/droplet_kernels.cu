@@ -231,8 +231,12 @@ droplet_rank_kernel(SysParams p, DropletOut o)
         }
         if (lane == 31) red[warp] = incl;
         __syncthreads();
-        uint32_t r = incl - sum;
-        for (int i = 0; i < warp; ++i) r += red[i];
+        uint32_t r = incl - sum, n = 0;
+        for (int i = 0; i < warps; ++i) {
+            r += i < warp ? red[i] : 0u;
+            n += red[i];
+        }
+        n = min(n, N);     // particles with tables: N, or fewer bits of a bitset that lacks some
         for (int i = c0; i < c1; ++i) {
             const uint32_t word = bits[i];
             base[i] = (IdxT)r;
@@ -241,14 +245,14 @@ droplet_rank_kernel(SysParams p, DropletOut o)
             for (uint32_t x = word; x; x &= x - 1u, ++r) {
                 const uint32_t b = (uint32_t)__ffs(x) - 1u, s = 32u * (uint32_t)i + b;
                 const bool row_start = s - __umulhi(s, p.magL) * L == 0u;
-                if (r < N) {
+                if (r < n) {
                     site[r] = (IdxT)s;
                     parent[r] = ((left >> b) & 1u) && !row_start ? r - 1u : r;
                 }
             }
         }
         __syncthreads();
-        for (uint32_t i = tid; i < N; i += T) {
+        for (uint32_t i = tid; i < n; i += T) {
             const uint32_t s = site[i];
             const uint32_t q = __umulhi(s, p.magL), x = s - q * L;
             uint32_t t[D];
@@ -272,7 +276,7 @@ droplet_rank_kernel(SysParams p, DropletOut o)
             for (int k = 0; k < D; ++k)
                 if (bond[k]) {
                     const uint32_t rt = rank_of(t[k]);
-                    if (rt < N) ok &= unite(parent, i, rt);
+                    if (rt < n) ok &= unite(parent, i, rt);
                 }
         }
         __syncthreads();
@@ -280,7 +284,7 @@ droplet_rank_kernel(SysParams p, DropletOut o)
         const uint32_t tail_words = (uint32_t)((sizeof(IdxT) * N + 3) / 4);
         for (uint32_t i = tid; i < tail_words; i += T) tail[i] = 0u;
         __syncthreads();
-        for (uint32_t i = tid; i < N; i += T) {
+        for (uint32_t i = tid; i < n; i += T) {
             const uint32_t root = find_root_ro(parent, i);
             // (two 16-bit counters per word; a count is below 65536)
             if constexpr (sizeof(IdxT) == 2) atomicAdd(tail + (root >> 1), 1u << ((root & 1u) << 4));

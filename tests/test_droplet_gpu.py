@@ -236,3 +236,25 @@ def test_droplets_of_two_contexts_in_turn():
             c.measure_droplets()
             _, occ, _ = chain.init_walkers(d, L, N, W, seed)
             assert c.largest_droplets(0).tolist() == [chain.largest_droplet(d, L, occ[w]) for w in range(W)]
+
+
+@pytest.mark.parametrize("desc", [(2, 20, 120, 40, 0, 0, 3), (3, 12, 300, 9, 0, 0, 4), (3, 48, 3000, 3, 0, 0, 5)])
+def test_droplets_of_restored_bitsets_that_lack_particles(desc):
+    """A restored state whose bitsets lack sites of the lists: the droplets of
+    the bits there are (no table entry is read that none has written)."""
+    d, L, N, W, _, _, seed = desc
+    words = (L ** d + 31) // 32
+    rng = np.random.default_rng(seed)
+    with m.Mucal([desc]) as mc:
+        ck = mc.checkpoint(0).copy()
+        at = 64                                       # the header's bytes
+        bits = ck[at:at + 4 * W * words].view(np.uint32).reshape(W, words)
+        _, occ, _ = chain.init_walkers(d, L, N, W, seed)
+        have = np.unpackbits(bits.view(np.uint8), axis=1, bitorder="little")[:, :L ** d]
+        np.testing.assert_array_equal(have, occ)
+        bits &= rng.integers(1 << 32, size=bits.shape, dtype=np.uint32)
+        bits[W - 1] = 0
+        mc.restore(0, ck)
+        mc.measure_droplets()
+        have = np.unpackbits(bits.view(np.uint8), axis=1, bitorder="little")[:, :L ** d]
+        assert mc.largest_droplets(0).tolist() == [chain.largest_droplet(d, L, have[w]) for w in range(W)]
