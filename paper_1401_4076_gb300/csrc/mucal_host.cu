@@ -135,7 +135,7 @@ void build_thresholds(const System &s, uint32_t *T)
     for (int b = 0; b < nb; ++b) {
         const double from = s.lnW[b];
         uint32_t *row = T + (size_t)b * s.p.tstride;
-        for (int j = width; j < s.p.tstride; ++j) row[j] = 0u;   // row padding, never read
+        for (int j = width; j < s.p.tstride; ++j) row[j] = 0u;   // refused: attempts past the end read it
         for (int j = 0; j < width; ++j) {
             const int to = b + (j - half);
             if (to < 0 || to >= nb) {
@@ -172,7 +172,8 @@ int ensure_thr_transposed(Context *c)
     for (auto &s : c->sys) {
         if (s.p.thrT) continue;
         const int pitch = (s.p.n_bins + 2 * mucal::kThrTPad + 3) & ~3;
-        const size_t bytes = (size_t)s.p.width * (size_t)pitch * sizeof(uint32_t);
+        // (the row behind the last stays zero, as the padding of the table's rows)
+        const size_t bytes = (size_t)(s.p.width + 1) * (size_t)pitch * sizeof(uint32_t);
         void *ptr = nullptr;
         CUDA_TRY(c, cudaMalloc(&ptr, bytes));
         s.p.thrT = static_cast<const uint32_t *>(ptr);

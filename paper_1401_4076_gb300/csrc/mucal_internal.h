@@ -28,10 +28,11 @@ struct SysParams {
     unsigned long long *hist;  // [rows][n_bins] histogram rows: one per walker (H_j(E)) when
                                // per-walker histograms are kept, else one per launch block
     int32_t hist_rows;         // rows in use for the current launch shape
-    const uint32_t *thr;       // [n_bins][tstride] acceptance thresholds (entries width..tstride-1
-                               // of a row unused)
-    const uint32_t *thrT;      // dE-major copy of the table, [width][thrT_pitch]: the threshold of
-                               // bin b at thrT[j * thrT_pitch + kThrTPad + b], zeros around it
+    const uint32_t *thr;       // [n_bins][tstride] acceptance thresholds; entries width..tstride-1
+                               // of a row are zero, and the rounds with several commits read
+                               // the first of them where a lane has no attempt
+    const uint32_t *thrT;      // dE-major copy of the table, [width + 1][thrT_pitch]: the threshold
+                               // of bin b at thrT[j * thrT_pitch + kThrTPad + b], zeros around it
                                // (NULL unless the launch shape's multi-commit rounds read it)
     int32_t thrT_pitch;
     unsigned long long *accepts; // [n_walkers] accepted moves in the last iteration

@@ -216,8 +216,8 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
     constexpr int NS = 2 * D;
     constexpr int TS = (4 * D + 1 + 3) & ~3;   // words of a table row (SysParams::tstride)
     constexpr bool PAIR = sizeof(IdxT) == 2;   // two list values fit one word
-    // dE + 2D of an attempt; one past the last, a row's padding, where T = 0,
-    // stands for an attempt past the end
+    // dE + 2D of an attempt; one past the last, where T = 0 (a row's padding, or
+    // the row behind the dE-major copy), stands for an attempt past the end
     constexpr uint32_t DEAD = 4 * D + 1;
     constexpr unsigned GMASK = W == 32 ? 0xffffffffu : ((1u << W) - 1u);
     const int lane = threadIdx.x & 31;
@@ -318,7 +318,9 @@ __device__ __forceinline__ void chain_scan(const SysParams &p, int w, bool activ
         uint32_t de = (uint32_t)(v.de(a, b, na, nb) + 2 * D);
 #pragma unroll
         for (int i = 0; i < NS; ++i) add_if_eq(de, 1u, na[i], b);    // (at most one of them)
-        code = place < near ? de : DEAD;
+        // (a state whose list and occupation disagree, as one may be restored, can
+        // give any dE: never a threshold outside the table)
+        code = place < near ? min(de, DEAD) : DEAD;
     };
     // The recurrence, and beside it, since its steps wait for one another,
     // the slots' random numbers two windows ahead.

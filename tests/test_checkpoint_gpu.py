@@ -84,3 +84,37 @@ def test_allocation_failure_is_reported_cleanly():
     with m.Mucal([(2, 8, 10, 4, 0, 0, 1)]) as ok:    # the device is still usable
         ok.run_iteration(5, 0)
         assert ok.histogram(0).sum() == 4 * 5 * 10
+
+
+@pytest.mark.parametrize("desc,launch", [
+    # the table staged, rows per walker, masks from global memory
+    ((2, 12, 40, 9, 0, 0, 4), dict(kernel=m.MUCAL_KERNEL_FIELD, lanes_per_walker=8, walkers_per_block=4)),
+    ((2, 90, 2501, 5, 0, 0, 7), dict(kernel=m.MUCAL_KERNEL_GROUP, lanes_per_walker=8, walkers_per_block=4)),
+    ((3, 17, 1201, 5, 0, 0, 8), dict(kernel=m.MUCAL_KERNEL_FIELD, lanes_per_walker=16, walkers_per_block=2)),
+    ((3, 30, 1201, 11, 0, 0, 9), dict(kernel=m.MUCAL_KERNEL_FIELD, lanes_per_walker=8, walkers_per_block=8)),
+    ((3, 30, 1201, 64, 0, 0, 9), dict(kernel=m.MUCAL_KERNEL_GROUP, lanes_per_walker=8, walkers_per_block=64)),
+], ids=lambda x: f"L{x[1]}-{x[3]}" if isinstance(x, tuple) else None)
+def test_rounds_on_a_restored_state_that_disagrees_with_itself(desc, launch):
+    """Lists with repeated sites and bitsets of other sites pass the restore's
+    checks.  The rounds with several commits then give no chain that means
+    anything, but count every attempt at an energy of the window."""
+    d, L, N, W, _, _, seed = desc
+    V = L ** d
+    words = (V + 31) // 32
+    rng = np.random.default_rng(seed)
+    with m.Mucal([desc]) as mc:
+        mc.set_launch(bits_in_smem=1, thr_window=0, multi_commit=1, **launch)
+        assert mc.launch()["multi_commit"] == 1
+        ck = mc.checkpoint(0).copy()
+        at = 64                                        # the header's bytes
+        bits = ck[at:at + 4 * W * words].view(np.uint32).reshape(W, words)
+        S = ck[at + 4 * W * words:at + 4 * W * words + 2 * W * V].view(np.uint16).reshape(W, V)
+        bits[:, :V // 32] = rng.integers(1 << 32, size=(W, V // 32), dtype=np.uint32)
+        S[:, ::2] = S[:, :1]
+        for beta in (0.0, 1.0):
+            mc.restore(0, ck)
+            mc.set_weights(0, -beta * np.arange(-d * N, 1, dtype=np.float64))
+            mc.run_iteration(3, 0)
+            assert mc.histogram(0).sum() == 3 * N * W
+            E = [mc.walker_state(0, w)[2] for w in range(W)]
+            assert min(E) >= -d * N and max(E) <= 0
