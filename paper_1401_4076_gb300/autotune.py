@@ -71,7 +71,8 @@ def autotune(systems, lnW=None, sweeps: int = 20, repeats: int = 3, cuda_stream=
                     mc.set_weights(i, w)
         it = 0
         seen = set()
-        for cfg in (cands or with_threshold_modes(candidates())):
+        # (the shape a new context has may be of a block size not listed)
+        for cfg in (cands or [mc.launch()] + with_threshold_modes(candidates())):
             try:
                 mc.set_launch(**cfg)
             except m.MucalError:

@@ -136,3 +136,18 @@ def test_default_launch_is_field_kernel_where_fields_fit():
         assert mc.launch()["kernel"] == m.MUCAL_KERNEL_GROUP
     with m.Mucal([(2, 16, 32, 8, 0, 0, 0), (3, 32, 3277, 8, 0, 0, 1)]) as mc:
         assert mc.launch()["kernel"] == m.MUCAL_KERNEL_GROUP
+
+
+def test_autotuner_times_the_default_shape():
+    """The shape a new context has is among those the autotuner times, also
+    where its block size is not one of the list."""
+    import torch
+    from paper_1401_4076_gb300.autotune import autotune, candidates
+    W = 100 * torch.cuda.get_device_properties(0).multi_processor_count
+    systems = [(2, 30, 100, W, 0, 0, 0)]
+    with m.Mucal(systems) as mc:
+        default = mc.launch()
+    assert not any(all(default[k] == c[k] for k in ("kernel", "lanes_per_walker", "walkers_per_block"))
+                   for c in candidates())
+    _, table = autotune(systems, sweeps=1, repeats=1)
+    assert any(cfg == default for cfg, _ in table)
