@@ -596,11 +596,30 @@ def measure(wl, args, systems, stream, device, world, flush, clocks_rank0=True, 
                                                           kernel_rate)
         except Exception as exc:   # reported, never fatal for the benchmark line
             roofline["latency_ceiling"] = {"error": repr(exc)[:200]}
-    # launches inside the timed region: per step one walker update and one
-    # histogram-reduce launch per system (the clears are driver memsets)
     return {"value": value, "ms_per_step": step_ms / args.steps, "roofline": roofline,
-            "clocks": clk, "gpu_launches": args.steps * (1 + n_sys),
+            "clocks": clk, "gpu_launches": args.steps * launches_per_step(systems, args.launch_desc),
             "acceptance": statistics.mean(accs)}
+
+
+def launches_per_step(systems, launch) -> int:
+    """Kernels of one timed step: the walker update and the histogram sum of all
+    systems (the clears are driver memsets), and per system, where the launch's
+    rounds with several commits read their thresholds from global memory, the
+    rewrite of the table copy they read."""
+    limit = 227 * 1024 - 2064        # a block's dynamic shared memory
+
+    def block_bytes(d, L, N, lo, hi, table):
+        bins = hi - lo + 1 if (lo, hi) != (0, 0) else d * N + 1
+        row = 48 if d == 2 else 64
+        V = L ** d
+        state = (V + 15) // 16 * 16 if launch["kernel"] == 2 else 4 * ((V + 31) // 32) * launch["bits_in_smem"]
+        w = launch["walkers_per_block"]
+        return w * state + (bins * row if table else 16 + w * (32 * row + 8))
+
+    fits = [all(block_bytes(d, L, N, lo, hi, table) <= limit for d, L, N, _, lo, hi, _ in systems)
+            for table in (True, False)]
+    masks = launch["multi_commit"] == 1 and not any(fits)
+    return 2 + (len(systems) if masks else 0)
 
 
 def latency_ceiling(systems, lnWs, launch, sweeps, stream, blocks_per_sm, sm_count, kernel_rate):

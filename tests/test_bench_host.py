@@ -98,3 +98,18 @@ def test_reference_arm_line(capsys):
     assert line["e2e"] == {"value": line["value"], "unit": "attempts/s",
                            "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}
     assert line["config"]["workload"] == wl.name
+
+
+def test_launches_of_a_timed_step():
+    """The walker update and one histogram sum whatever the number of systems;
+    a table copy per system where the rounds read masks from it."""
+    from paper_1401_4076_gb300 import workloads
+    group = dict(kernel=1, lanes_per_walker=8, walkers_per_block=28, bits_in_smem=1, persistent=0,
+                 thr_window=0, multi_commit=1)
+    batch = workloads.batched_uneven().systems
+    assert bench.launches_per_step(workloads.MEDIUM_2D.systems, group) == 2        # table staged
+    assert bench.launches_per_step(workloads.LARGE_3D.systems, group) == 2         # rows per walker
+    assert bench.launches_per_step(batch, dict(group, lanes_per_walker=16, walkers_per_block=4)) == 2
+    assert bench.launches_per_step(batch, dict(group, lanes_per_walker=16, walkers_per_block=24)) == 2 + 27
+    assert bench.launches_per_step(batch, dict(group, walkers_per_block=4, multi_commit=0)) == 2
+    assert bench.launches_per_step(workloads.LARGE_3D.systems, dict(group, kernel=2, walkers_per_block=4)) == 2
