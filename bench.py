@@ -55,27 +55,19 @@ def alg_ops_per_attempt(d: int) -> int:
 
 
 # DRAM bytes (read + write) of one walker-update launch of a workload's
-# default iteration, from the one-pass ncu capture summarised under profiles/,
-# valid only for the launch shape and the kernel source it was taken with
-# (sha256 prefix of walker_chain.cuh); any other shape or any change to the
-# kernel makes the figure stale (null).  The persistent flag is not part of
-# the shape here: when every block is resident at once (147 blocks of 28
-# walkers on 152 SMs) the persistent launch runs the same blocks.
+# default iteration, from the ncu captures summarised under profiles/, valid
+# only for the launch shape and the kernel source it was taken with (sha256
+# prefix, see _kernel_sha); any other shape or any change to the kernel makes
+# the figure stale (null).  The persistent flag is not part of the shape here:
+# when every block is resident at once (147 blocks of 28 walkers on 152 SMs) the
+# persistent launch runs the same blocks.  Rounds with one commit, of an earlier
+# kernel source (the 3D list's first record: with several commits, before the
+# sliding window):
 TRAFFIC_MEASURED = {
     # one full 1000-sweep launch (profiles/walker_update_field_2d-L64-N410-w4096.md)
     "2d-L64-N410-w4096": {"bytes": 34.239e6 + 802.815e6, "kernel_sha": "4f112a9b4d61e7f4",
                           "launch": {"kernel": 2, "lanes_per_walker": 8, "walkers_per_block": 28,
                                      "thr_window": 0, "multi_commit": 0}},
-    # one full 200-sweep launch (profiles/walker_update_group_batched-27-systems-w16384.md)
-    # (and the multi-commit shape the autotuner also picks there, by under 1 %)
-    "batched-27-systems-w16384": [
-        {"bytes": 704.779e9 + 300.284e9, "kernel_sha": "4f112a9b4d61e7f4",
-         "launch": {"kernel": 1, "lanes_per_walker": 16, "bits_in_smem": 1, "thr_window": 0,
-                    "multi_commit": 0}},
-        {"bytes": 761.331e9 + 317.758e9, "kernel_sha": "4f112a9b4d61e7f4",
-         "launch": {"kernel": 1, "lanes_per_walker": 8, "bits_in_smem": 1, "thr_window": 0,
-                    "multi_commit": 1}},
-    ],
     # a 5-sweep launch scaled by 40 to the workload's 200 sweeps (the list reads and
     # writes grow with the attempts; profiles/walker_update_group_3d-L32-N3277-w8192.md),
     # with multi-commit rounds and with one commit per round
@@ -89,53 +81,78 @@ TRAFFIC_MEASURED = {
     ],
 }
 
-# Executed instructions per attempted move of the walker-update kernel, from
-# one ncu capture of a launch of the workload (smsp__inst_executed.sum x 32
-# and smsp__thread_inst_executed.sum, divided by the launch's attempts), under
-# the same validity rule as the traffic record: launch shape and kernel source.
-INSTR_MEASURED = {
-    # the full 1000-sweep launch of the traffic record
-    "2d-L64-N410-w4096": {"warp_inst_per_attempt": 4.0031106e10 / 1.67936e9,
-                          "thread_inst_per_attempt": 1.0419877e12 / 1.67936e9,
-                          "kernel_sha": "4f112a9b4d61e7f4",
-                          "launch": {"kernel": 2, "lanes_per_walker": 8, "thr_window": 0,
-                                     "multi_commit": 0}},
-    # 2-sweep launch, same shape as the traffic record (instructions per attempt do not
-    # depend on the sweep count beyond the per-block set-up)
-    "batched-27-systems-w16384": [
-        {"warp_inst_per_attempt": 4.215209e9 / 72.3314e6,
-         "thread_inst_per_attempt": 1.21995e11 / 72.3314e6,
-         "kernel_sha": "4f112a9b4d61e7f4", "any_sweeps": True,
-         "launch": {"kernel": 1, "lanes_per_walker": 16, "bits_in_smem": 1, "thr_window": 0,
-                    "multi_commit": 0}},
-        {"warp_inst_per_attempt": 3.788915e9 / 72.3314e6,
-         "thread_inst_per_attempt": 1.0942e11 / 72.3314e6,
-         "kernel_sha": "4f112a9b4d61e7f4", "any_sweeps": True,
-         "launch": {"kernel": 1, "lanes_per_walker": 8, "bits_in_smem": 1, "thr_window": 0,
+# and rounds with several commits (profiles/walker_update_scan.md): the 2D launch
+# in full, the others 20-sweep launches scaled by 10 to the workloads' 200 sweeps
+# (the list reads and writes grow with the attempts).
+TRAFFIC_SEVERAL = {
+    "2d-L64-N410-w4096": [
+        {"bytes": 33.901e6 + 964.945e6, "kernel_sha": "55f1c14ab48d0cdb",
+         "launch": {"kernel": 2, "lanes_per_walker": 8, "walkers_per_block": 28, "thr_window": 0,
                     "multi_commit": 1}},
+        {"bytes": 36.000e6 + 759.821e6, "kernel_sha": "55f1c14ab48d0cdb",
+         "launch": {"kernel": 1, "lanes_per_walker": 8, "walkers_per_block": 28, "bits_in_smem": 1,
+                    "thr_window": 0, "multi_commit": 1}},
+    ],
+    "batched-27-systems-w16384": [
+        {"bytes": 10 * (72.867e9 + 29.770e9), "kernel_sha": "55f1c14ab48d0cdb",
+         "launch": {"kernel": 1, "lanes_per_walker": 16, "walkers_per_block": 24, "bits_in_smem": 1,
+                    "thr_window": 0, "multi_commit": 1}},
     ],
     "3d-L32-N3277-w8192": [
-        {"warp_inst_per_attempt": 4.781667e9 / 134.2259e6,
-         "thread_inst_per_attempt": 1.426715e11 / 134.2259e6,
-         "kernel_sha": "4f112a9b4d61e7f4", "any_sweeps": True,
-         "launch": {"kernel": 1, "lanes_per_walker": 4, "bits_in_smem": 1, "thr_window": 0,
+        {"bytes": 10 * (43.974e9 + 22.919e9), "kernel_sha": "55f1c14ab48d0cdb",
+         "launch": {"kernel": 1, "lanes_per_walker": 8, "walkers_per_block": 28, "bits_in_smem": 1,
+                    "thr_window": 0, "multi_commit": 1}},
+    ],
+}
+
+# Executed instructions per attempted move of the walker-update kernel, from
+# the same launches (smsp__inst_executed.sum and
+# smsp__thread_inst_executed.sum, divided by the launch's attempts), under the
+# same validity rule as the traffic record: launch shape and kernel source.
+# They do not depend on the sweep count beyond the per-block set-up.
+INSTR_SEVERAL = {
+    "2d-L64-N410-w4096": [
+        {"warp_inst_per_attempt": 30.507945e9 / 1.67936e9,
+         "thread_inst_per_attempt": 9.440676e11 / 1.67936e9, "kernel_sha": "55f1c14ab48d0cdb",
+         "launch": {"kernel": 2, "lanes_per_walker": 8, "walkers_per_block": 28, "thr_window": 0,
                     "multi_commit": 1}},
-        {"warp_inst_per_attempt": 2.974781e9 / 134.2259e6,
-         "thread_inst_per_attempt": 8.90372e10 / 134.2259e6,
-         "kernel_sha": "4f112a9b4d61e7f4", "any_sweeps": True,
-         "launch": {"kernel": 1, "lanes_per_walker": 4, "bits_in_smem": 1, "thr_window": 0,
-                    "multi_commit": 0}},
+        {"warp_inst_per_attempt": 30.501918e9 / 1.67936e9,
+         "thread_inst_per_attempt": 9.551687e11 / 1.67936e9, "kernel_sha": "55f1c14ab48d0cdb",
+         "launch": {"kernel": 1, "lanes_per_walker": 8, "walkers_per_block": 28, "bits_in_smem": 1,
+                    "thr_window": 0, "multi_commit": 1}},
+    ],
+    "batched-27-systems-w16384": [
+        {"warp_inst_per_attempt": 21.635541e9 / 7.2331402e8,
+         "thread_inst_per_attempt": 6.704859e11 / 7.2331402e8, "kernel_sha": "55f1c14ab48d0cdb", "any_sweeps": True,
+         "launch": {"kernel": 1, "lanes_per_walker": 16, "walkers_per_block": 24, "bits_in_smem": 1,
+                    "thr_window": 0, "multi_commit": 1}},
+    ],
+    "3d-L32-N3277-w8192": [
+        {"warp_inst_per_attempt": 11.874410e9 / 5.3690368e8,
+         "thread_inst_per_attempt": 3.659246e11 / 5.3690368e8, "kernel_sha": "55f1c14ab48d0cdb", "any_sweeps": True,
+         "launch": {"kernel": 1, "lanes_per_walker": 8, "walkers_per_block": 28, "bits_in_smem": 1,
+                    "thr_window": 0, "multi_commit": 1}},
     ],
 }
 
 KERNEL_NAMES = {0: "walker_update_thread", 1: "walker_update_group", 2: "walker_update_field"}
 
 
-def _kernel_sha() -> str:
+def kernel_name(launch: dict) -> str:
+    if launch.get("multi_commit"):
+        return "walker_update_scan"
+    return KERNEL_NAMES.get(launch.get("kernel"), "walker_update")
+
+
+def _kernel_sha(several: bool = False) -> str:
     import hashlib
-    # the walker-update kernels are compiled from walker_chain.cuh
-    with open(os.path.join(ROOT, "paper_1401_4076_gb300", "csrc", "walker_chain.cuh"), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    # the walker-update kernels are compiled from walker_chain.cuh, those with
+    # several commits per round from walker_scan.cuh too
+    h = hashlib.sha256()
+    for name in ("walker_chain.cuh", "walker_scan.cuh")[:2 if several else 1]:
+        with open(os.path.join(ROOT, "paper_1401_4076_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def _record_for(table: dict, workload: str, sweeps_default: bool, launch: dict):
@@ -148,16 +165,17 @@ def _record_for(table: dict, workload: str, sweeps_default: bool, launch: dict):
         # the launch keys a record names must match (records name the kernel,
         # the lanes per walker, the bitset staging, the threshold mode and the
         # rounds; the split into blocks does not change the per-attempt work
-        # or access pattern)
+        # or access pattern of rounds with one commit)
         if any(launch.get(k) != v for k, v in rec["launch"].items()):
             continue
-        if _kernel_sha() == rec["kernel_sha"]:
+        if _kernel_sha(bool(rec["launch"].get("multi_commit"))) == rec["kernel_sha"]:
             return rec
     return None
 
 
 def _measured_traffic(workload: str, sweeps_default: bool, launch: dict):
-    rec = _record_for(TRAFFIC_MEASURED, workload, sweeps_default, launch)
+    table = TRAFFIC_SEVERAL if launch.get("multi_commit") else TRAFFIC_MEASURED
+    rec = _record_for(table, workload, sweeps_default, launch)
     return None if rec is None else rec["bytes"]
 
 
@@ -572,7 +590,7 @@ def measure(wl, args, systems, stream, device, world, flush, clocks_rank0=True, 
                 "unit": "Tops/s", "frac": achieved / peak_ops,
                 "traffic": _measured_traffic(wl.name, sweeps == wl.sweeps, args.launch_desc),
                 "peak_source": f"{sm_count} SMs x 128 lanes x {f_mhz} MHz ({peak_kind} max clock)",
-                "kernel": KERNEL_NAMES.get(args.launch_desc.get("kernel"), "walker_update"),
+                "kernel": kernel_name(args.launch_desc),
                 "kernel_ms": k_ms,
                 "kernel_attempts_per_s": kernel_rate,
                 "alg_ops_per_attempt": alg_ops_per_attempt(d_max),
@@ -580,12 +598,12 @@ def measure(wl, args, systems, stream, device, world, flush, clocks_rank0=True, 
                                  "threshold 1 + histogram 1",
                 "chains_per_sm": sum(s[3] for s in systems) / sm_count,
                 "resident_blocks_per_sm": blocks_per_sm}
-    rec = _record_for(INSTR_MEASURED, wl.name, sweeps == wl.sweeps, args.launch_desc)
+    rec = _record_for(INSTR_SEVERAL, wl.name, sweeps == wl.sweeps, args.launch_desc)
     if rec is not None:
         # issue slots: 4 warp instructions per SM and clock
         roofline["issue"] = {"warp_inst_per_attempt": rec["warp_inst_per_attempt"],
                              "thread_inst_per_attempt": rec["thread_inst_per_attempt"],
-                             "frac": kernel_rate * rec["warp_inst_per_attempt"] / 32.0
+                             "frac": kernel_rate * rec["warp_inst_per_attempt"]
                              / (sm_count * 4 * f_mhz * 1e6)}
     lnWs = [mc.weights(s) for s in range(n_sys)]
     mc.close()

@@ -113,3 +113,40 @@ def test_launches_of_a_timed_step():
     assert bench.launches_per_step(batch, dict(group, lanes_per_walker=16, walkers_per_block=24)) == 2 + 27
     assert bench.launches_per_step(batch, dict(group, walkers_per_block=4, multi_commit=0)) == 2
     assert bench.launches_per_step(workloads.LARGE_3D.systems, dict(group, kernel=2, walkers_per_block=4)) == 2
+
+
+def test_records_of_rounds_with_several_commits(monkeypatch):
+    """Their records stand for both kernel sources and are found by the launch;
+    the line names their kernel and the issue slots they use."""
+    launch = {"kernel": 1, "lanes_per_walker": 8, "multi_commit": 1}
+    rec = {"launch": dict(launch), "kernel_sha": bench._kernel_sha(True), "bytes": 5.0}
+    assert bench._kernel_sha(True) != bench._kernel_sha()
+    monkeypatch.setattr(bench, "TRAFFIC_SEVERAL", {"x": [rec]})
+    assert bench._measured_traffic("x", True, dict(launch, persistent=1)) == 5.0
+    assert bench._measured_traffic("x", True, dict(launch, multi_commit=0)) is None
+    assert bench._measured_traffic("x", False, launch) is None
+    rec["kernel_sha"] = bench._kernel_sha()              # walker_chain.cuh alone is not enough
+    assert bench._measured_traffic("x", True, launch) is None
+    assert bench.kernel_name(launch) == "walker_update_scan"
+    assert bench.kernel_name(dict(launch, multi_commit=0)) == "walker_update_group"
+    assert bench.kernel_name({"kernel": 0, "multi_commit": 0}) == "walker_update_thread"
+
+
+def test_stored_records_of_rounds_with_several_commits():
+    """The stored ones name one launch each and hold what an attempt can need:
+    a few hundred bytes, tens of warp instructions of 32 lanes or fewer."""
+    from paper_1401_4076_gb300 import workloads
+    attempts = {w.name: w.attempts_per_iteration()
+                for w in (workloads.MEDIUM_2D, workloads.LARGE_3D, workloads.batched_uneven())}
+    for table in (bench.TRAFFIC_SEVERAL, bench.INSTR_SEVERAL):
+        assert set(table) == set(attempts)
+        for name, recs in table.items():
+            keys = [tuple(sorted(r["launch"].items())) for r in recs]
+            assert len(set(keys)) == len(keys)
+            for r in recs:
+                assert r["launch"]["multi_commit"] == 1 and len(r["kernel_sha"]) == 16
+                if "bytes" in r:
+                    assert r["bytes"] / attempts[name] < 300
+                else:
+                    ratio = r["thread_inst_per_attempt"] / r["warp_inst_per_attempt"]
+                    assert 10 < r["warp_inst_per_attempt"] < 60 and 20 < ratio <= 32
